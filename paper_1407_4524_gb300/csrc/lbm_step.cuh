@@ -115,8 +115,14 @@ __device__ __forceinline__ double feq_x(const Params &p, int i, double rho, cons
     return w * rho * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * usq);
 }
 
+// not an infinity and not a NaN (integer test: the FP64 pipe is the scarce one)
+__device__ __forceinline__ bool finite_x(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
+// moments and relaxation with every product written out: the form of the
+// formulas, kept for nodes whose populations or velocity are not finite (where
+// 0 * inf is NaN, so leaving products with 0 out would change the result)
 template <class L>
-__device__ __forceinline__ void moments_x(const Params &p, const double f[], double &rho, double u[3]) {
+__device__ __forceinline__ void moments_all_x(const Params &p, const double f[], double &rho, double u[3]) {
     double r = 0.0, j0 = 0.0, j1 = 0.0, j2 = 0.0;
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
@@ -138,7 +144,7 @@ __device__ __forceinline__ void moments_x(const Params &p, const double f[], dou
 }
 
 template <class L>
-__device__ __forceinline__ void collide_x(const Params &p, double f[], double rho, const double u[3]) {
+__device__ __forceinline__ void collide_all_x(const Params &p, double f[], double rho, const double u[3]) {
     const double omega = p.omega;
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
@@ -152,6 +158,113 @@ __device__ __forceinline__ void collide_x(const Params &p, double f[], double rh
             v = v + (1.0 - 0.5 * omega) * L::template w<double>(i) * (3.0 * (cg - ug) + 9.0 * cu * cg);
         }
         f[i] = v;
+    }
+}
+
+// The FP64 mode is bound by the FP64 pipe (2 lanes per clock and SM: 0.63e12
+// instructions a second on the chip), so both functions issue only the
+// operations that can change the result.  Left out: products with 0 and +-1
+// (x + 0 * y = x for finite y), the division by and product with rho0 = 1, and
+// whatever the two directions i, opp(i) of a pair share (c_o . u = -(c_i . u)
+// exactly: rounding to nearest is symmetric).  Every remaining operation and
+// its order are those of the *_all_x forms, so the results are the same bits.
+// D3Q19: 216 FP64 operations a node instead of 437 and three divisions; the
+// 256x128x128 sphere channel's step 3.66 -> 2.49 ms, the 200x80 cylinder
+// channel's 38.8 -> 31.0 us.
+template <class L>
+__device__ __forceinline__ void moments_x(const Params &p, const double f[], double &rho, double u[3]) {
+    double r = 0.0, j[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+        const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
+        r += f[i];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (c[a] == 1) j[a] += f[i];
+            if (c[a] == -1) j[a] -= f[i];
+        }
+    }
+    if (p.has_force)
+        for (int a = 0; a < 3; ++a) j[a] += 0.5 * p.g[a];
+    if (p.eq != 0 || p.rho0 != 1.0) {
+        const double den = p.eq == 0 ? p.rho0 : r;
+        for (int a = 0; a < 3; ++a) j[a] = j[a] / den;
+    }
+    rho = r;
+    for (int a = 0; a < 3; ++a) u[a] = j[a];
+    if (!(finite_x(r) && finite_x(u[0]) && finite_x(u[1]) && finite_x(u[2]))) moments_all_x<L>(p, f, rho, u);
+}
+
+// c_i . v without the products with 0 and +-1 (v finite)
+template <class L> __device__ __forceinline__ double cdot_x(int i, const double v[3]) {
+    const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
+    double s = 0.0;
+    bool any = false;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (c[a] == 0) continue;
+        s = any ? (c[a] > 0 ? s + v[a] : s - v[a]) : (c[a] > 0 ? v[a] : -v[a]);
+        any = true;
+    }
+    return s;
+}
+
+// EQ: 0 quasi-incompressible with rho0 = 1, 1 with any rho0, 2 standard
+template <class L, int EQ, bool FORCE>
+__device__ __forceinline__ void collide_pairs_x(const Params &p, double f[], double rho, const double u[3]) {
+    const double omega = p.omega;
+    double usq = u[0] * u[0] + u[1] * u[1];
+    if constexpr (L::D == 3 || FORCE) usq = usq + u[2] * u[2]; // (2-D, no force: u_z = 0)
+    const double h = 1.5 * usq;
+    double ug = 0.0;
+    if constexpr (FORCE) ug = u[0] * p.g[0] + u[1] * p.g[1] + u[2] * p.g[2];
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+        const int o = L::opp(i);
+        if (o < i) continue; // relaxed with its partner
+        const double w = L::template w<double>(i);
+        const double cu = cdot_x<L>(i, u);
+        const double t3 = 3.0 * cu, t45 = 4.5 * cu * cu;
+        double cg = 0.0, cc = 0.0;
+        if constexpr (FORCE) {
+            cg = cdot_x<L>(i, p.g);
+            cc = 9.0 * cu * cg; // the same for both directions
+        }
+#pragma unroll
+        for (int k = 0; k < (i == 0 ? 1 : 2); ++k) {
+            const int d = k == 0 ? i : o;
+            double feq;
+            if constexpr (EQ == 2) {
+                const double s = i == 0 ? 1.0 : ((k == 0 ? 1.0 + t3 : 1.0 - t3) + t45);
+                feq = w * rho * (s - h);
+            } else {
+                const double s = i == 0 ? -h : ((k == 0 ? t3 + t45 : t45 - t3) - h);
+                feq = w * (rho + (EQ == 0 ? s : p.rho0 * s));
+            }
+            const double fi = f[d];
+            double v = fi - omega * (fi - feq);
+            if constexpr (FORCE)
+                v = v + (1.0 - 0.5 * omega) * w * (3.0 * ((k == 0 ? cg : -cg) - ug) + cc);
+            f[d] = v;
+        }
+    }
+}
+
+template <class L>
+__device__ __forceinline__ void collide_x(const Params &p, double f[], double rho, const double u[3]) {
+    bool fin = finite_x(u[0]) && finite_x(u[1]) && finite_x(u[2]);
+    if (p.has_force) fin = fin && finite_x(p.g[0]) && finite_x(p.g[1]) && finite_x(p.g[2]);
+    if (!fin) {
+        collide_all_x<L>(p, f, rho, u);
+    } else if (p.has_force) {
+        if (p.eq != 0) collide_pairs_x<L, 2, true>(p, f, rho, u);
+        else collide_pairs_x<L, 1, true>(p, f, rho, u);
+    } else if (p.eq != 0) {
+        collide_pairs_x<L, 2, false>(p, f, rho, u);
+    } else if (p.rho0 != 1.0) {
+        collide_pairs_x<L, 1, false>(p, f, rho, u);
+    } else {
+        collide_pairs_x<L, 0, false>(p, f, rho, u);
     }
 }
 
