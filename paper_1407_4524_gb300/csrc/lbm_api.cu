@@ -4,15 +4,13 @@
 // buffers (rho,u at the nodes flagged FL_MAC), the node flags, two owner
 // arrays (solid owner at t and t+1), two cut-link buffers (t and t+1), the
 // per-link momentum-exchange contributions, the covered/uncovered lists and
-// the force/torque ring.  lbm_step enqueues, per step, in FP64 mode:
-//   moving bodies only: k_prep (poses, link prefixes),
-//                       k_geom_a, k_geom_b, k_geom_c  (geometry of t+1)
-//   k_links (wall values + ME per link), k_bulk (stream-collide; then
-//   k_zouhe for the Zou-He face nodes), k_finish (per-body series row;
-//   A+/A- impulsive terms and refill), k_free (free bodies);
-// in the reduced-precision modes (do_step_overlapped): k_fprep on the main
-// stream, then the surface kernels (k_fgeom1/2, k_bnd, k_finish, k_free) on
-// a high-priority side stream beside k_bulk (+ k_zouhe) on the main stream.
+// the force/torque ring.  lbm_step enqueues, per step (do_step):
+//   main stream: k_prep / k_fprep (poses, solid flags, link prefixes), k_links
+//   (wall values + ME per link), k_bulk / k_bulk_pair (stream-collide; then
+//   k_zouhe for the Zou-He face nodes);
+//   high-priority side stream, beside the stream-collide pass: k_geom_a/b/c or
+//   k_fgeom1/2l (geometry of t+1, moving bodies), k_finish (per-body series
+//   row; A+/A- impulsive terms and refill), k_free (free bodies).
 // Each lbm_step call ends with a step event that the series reads wait on.
 // The serving batch (lbm_batch_*) keeps solves of this kind in slots and
 // replays a CUDA graph of batched ticks (lbm_batch.cu).  Every persistent
@@ -495,7 +493,12 @@ GeomArgs geom_args(lbm_domain *D, bool moving_step) {
     g.bn_mov_cnt = D->bn_cnt + 1 + nxt;
     g.bn_static_cap = D->bn_static_cap;
     g.bn_mov_cap = D->bn_mov_cap;
-    g.do_flags = (moving_step && D->prec == LBM_FP64) ? 1 : 0;
+    // FP64 mode, semi-implicit schemes (one stream): the node flags follow the
+    // geometry; elsewhere the kept-moment band only gains flags (linkmode, or
+    // geom_a in FP64 mode)
+    const bool semi = D->n_free && D->p.free_scheme != LBM_FREE_EXPLICIT;
+    g.do_flags = (moving_step && D->prec == LBM_FP64 && semi) ? 1 : 0;
+    g.do_band = (moving_step && D->prec == LBM_FP64 && !semi) ? 1 : 0;
     return g;
 }
 
@@ -546,8 +549,6 @@ int upload_bodies(lbm_domain *D) {
     return LBM_OK;
 }
 
-int do_step_overlapped(lbm_domain *D);
-
 // reduced-precision modes: boundary-node lists of step t from scratch
 int build_bnd_lists(lbm_domain *D) {
     if (D->p.linkmode) { // link mode keeps cut-link lists instead
@@ -594,6 +595,8 @@ int timing_events(lbm_domain *D, cudaEvent_t &a, cudaEvent_t &b) {
 // the free-body scheme a step runs (the explicit one when no body is free)
 int step_scheme(const lbm_domain *D) { return D->n_free ? D->p.free_scheme : LBM_FREE_EXPLICIT; }
 
+int geometry(lbm_domain *D, const GeomArgs &g, bool links, cudaStream_t s);
+
 // semi-implicit schemes, after the stream-collide pass: the force row of step
 // t (with the impulsive terms of the previous displacement, or of the
 // predicted one whose lists sb_pred names), the velocities of t+1, the poses
@@ -614,15 +617,8 @@ int finish_semi(lbm_domain *D, int scheme, const StepBufs &sb) {
     const unsigned long long *tdev = D->counters + 9 + (D->t & 1);
     CK(launch_free(D->p, D->dbodies, D->series, D->counters, tdev, D->s));
     CK(launch_pose1(D->p, D->dbodies, D->poses, tdev, D->s));
-    GeomArgs g = geom_args(D, true);
-    if (prec == LBM_FP64) {
-        CK(launch_geom_a(Q, D->p, g, D->s));
-        CK(launch_geom_b(Q, D->p, g, D->s));
-        CK(launch_geom_c(Q, D->p, g, D->s));
-    } else {
-        CK(launch_fgeom1(Q, D->p, g, D->s));
-        CK(launch_fgeom2(Q, D->p, g, D->s));
-    }
+    int rc = geometry(D, geom_args(D, true), true, D->s);
+    if (rc) return rc;
     StepBufs s2 = sb;
     s2.phase = scheme == LBM_FREE_AIDUN ? PH_IMP : PH_FIX;
     CK(launch_finish(Q, prec, D->p, s2, D->s));
@@ -639,157 +635,101 @@ GeomArgs predicted_geom(lbm_domain *D) {
     return g;
 }
 
+// the stream-collide pass on the main stream, between the timing events
+int bulk_pass(lbm_domain *D, const StepBufs &sb) {
+    cudaEvent_t ta = nullptr, tb = nullptr;
+    if (D->timing) {
+        int trc = timing_events(D, ta, tb);
+        if (trc) return trc;
+        CK(record_timing(D, ta));
+    }
+    CK(launch_bulk(D->Q, D->prec, D->p, sb, D->s));
+    if (D->timing) CK(record_timing(D, tb));
+    return LBM_OK;
+}
+
+void step_done(lbm_domain *D) {
+    D->t += 1;
+    if (D->capturing) D->cap_k += 1;
+}
+
+// poses of t and t+1, the solid flags of t, the prefixes of the cut-link lists
+int prepare_step(lbm_domain *D) {
+    const int cur = (int)(D->t & 1), nxt = cur ^ 1;
+    const unsigned long long *tdev = D->counters + 9 + cur;
+    if (D->prec == LBM_FP64) {
+        // (the A+/A- lists of the previous step update the solid flags)
+        if (D->n_moving || D->prep_dirty)
+            CK(launch_prep(D->p, D->dbodies, D->link_cnt[cur], D->link_pre, D->tile_pre, D->poses, D->t, tdev, D->flags,
+                           D->apm_cnt, D->apm_cell, D->apm_sign, D->s));
+    } else if (D->n_moving || D->prep_dirty || D->lists_dirty) {
+        CK(launch_fprep(D->p, D->dbodies, D->poses, D->t, tdev, D->flags, D->chg_cnt, D->chg_cell, D->chg_val,
+                        D->chg_cap, D->apm_cnt, D->bn_cnt + 1 + nxt, D->link_cnt[cur], D->link_cnt[nxt], D->tile_pre,
+                        D->s));
+    }
+    D->prep_dirty = false;
+    D->lists_dirty = false;
+    return LBM_OK;
+}
+
+// owners, covered / uncovered lists and cut links of t+1 (moving bodies)
+int geometry(lbm_domain *D, const GeomArgs &g, bool links, cudaStream_t s) {
+    if (D->prec == LBM_FP64) {
+        CK(launch_geom_a(D->Q, D->p, g, s));
+        CK(launch_geom_b(D->Q, D->p, g, s));
+        if (links) CK(launch_geom_c(D->Q, D->p, g, s));
+    } else {
+        CK(launch_fgeom1(D->Q, D->p, g, s));
+        if (links) CK(launch_fgeom2(D->Q, D->p, g, s));
+    }
+    return LBM_OK;
+}
+
+// semi-implicit free-body schemes: the geometry of t+1 follows the force of
+// t, so the whole step runs on one stream
+int step_semi(lbm_domain *D, int scheme) {
+    int rc;
+    if (D->prec == LBM_FP64) {
+        // node flags of t+1 (moments kept on a band around the free bodies) from
+        // the displacement with U(t), and scheme 2's predicted lists
+        const GeomArgs g = scheme == LBM_FREE_PREDICTOR ? predicted_geom(D) : geom_args(D, true);
+        if ((rc = geometry(D, g, false, D->s))) return rc;
+    } else if (scheme == LBM_FREE_PREDICTOR) {
+        CK(cudaMemsetAsync(D->apm_pred_cnt, 0, sizeof(long long) * (size_t)D->nb, D->s));
+        if ((rc = geometry(D, predicted_geom(D), false, D->s))) return rc;
+    }
+    StepBufs sb = step_bufs(D);
+    CK(launch_links(D->Q, D->prec, D->p, sb, D->links_grid, D->s));
+    if ((rc = bulk_pass(D, sb))) return rc;
+    if ((rc = finish_semi(D, scheme, sb))) return rc;
+    step_done(D);
+    return LBM_OK;
+}
+
+// One step.  Stream s: prep -> cut links (wall values into the solid nodes'
+// slots, momentum exchange) -> stream-collide of every fluid node (moments
+// kept at the nodes near bodies).  Side stream: after prep, the owners,
+// covered / uncovered lists and cut links of t+1 of the moving bodies; after
+// the cut links, the end of step (series row, impulsive terms with covered
+// nodes re-pulled from fhat(t) and its wall values, refill of uncovered nodes)
+// and the free-body update.  The side stream overlaps the stream-collide pass
+// and touches no data it reads or writes: the links of t+1 go to the other
+// list buffer, the kept-moment band only gains flags, solid flags change in
+// the next prep, refilled nodes were solid at t.  In FP64 mode this hides the
+// sequential link sums (0.68 ms for the 9.6k links of the 256x128x128 sphere
+// channel, whose stream-collide pass takes 1.80 ms: step 2.49 -> 1.84 ms).
 int do_step(lbm_domain *D) {
     const int Q = D->Q, prec = D->prec;
-    if (prec != LBM_FP64 && D->nb) return do_step_overlapped(D);
-    D->lists_dirty = false; // boundary-node lists belong to the overlapped path only
-    const int scheme = step_scheme(D);
-    if (D->nb && (D->n_moving || D->prep_dirty)) {
-        // the A+/A- lists of the previous step update the solid flags of t
-        CK(launch_prep(D->p, D->dbodies, D->link_cnt[D->t & 1], D->link_pre, D->tile_pre, D->poses, D->t,
-                       D->counters + 9 + (D->t & 1), D->flags, D->apm_cnt, D->apm_cell, D->apm_sign, D->s));
-        D->prep_dirty = false;
-    }
-    if (D->n_moving) {
-        // semi-implicit schemes: the node flags of t+1 (moments kept on a band
-        // around the free bodies) from the displacement with U(t), and scheme
-        // 2's predicted lists; the cut links follow the displacement made
-        GeomArgs g = scheme == LBM_FREE_PREDICTOR ? predicted_geom(D) : geom_args(D, true);
-        CK(launch_geom_a(Q, D->p, g, D->s));
-        CK(launch_geom_b(Q, D->p, g, D->s));
-        if (scheme == LBM_FREE_EXPLICIT) CK(launch_geom_c(Q, D->p, g, D->s));
-    }
-    StepBufs sb = step_bufs(D);
-    if (D->nb) CK(launch_links(Q, prec, D->p, sb, D->links_grid, D->s));
-    cudaEvent_t ta = nullptr, tb = nullptr;
-    if (D->timing) {
-        int trc = timing_events(D, ta, tb);
-        if (trc) return trc;
-        CK(record_timing(D, ta));
-    }
-    CK(launch_bulk(Q, prec, D->p, sb, D->s));
-    if (D->timing) CK(record_timing(D, tb));
-    if (scheme != LBM_FREE_EXPLICIT) {
-        int rc = finish_semi(D, scheme, sb);
-        if (rc) return rc;
-    } else {
-        if (D->nb) CK(launch_finish(Q, prec, D->p, sb, D->s));
-        if (D->n_free) CK(launch_free(D->p, D->dbodies, D->series, D->counters, D->counters + 9 + (D->t & 1), D->s));
-    }
-    D->t += 1;
-    if (D->capturing) D->cap_k += 1;
-    return LBM_OK;
-}
-
-// Reduced-precision modes.  Stream s: prep -> bulk (every fluid node that is
-// not a boundary node).  Side stream, after prep: owner and flag changes of
-// t+1 (moving bodies), the boundary-node kernel (cut links, momentum
-// exchange, collision of the boundary nodes) and the end-of-step kernel
-// (series row, impulsive terms, refill).  The bulk kernel reads fhat(t) and
-// the flags of t and writes fhat(t+1) of the non-boundary fluid nodes; the
-// side stream writes fhat(t+1) of the boundary and refilled nodes, the owner
-// array of t+1, the lists and the accumulators: the two streams touch
-// disjoint data.  Flag changes are applied by the next prep.
-int do_step_links(lbm_domain *D);
-
-int do_step_overlapped(lbm_domain *D) {
-    if (D->p.linkmode) return do_step_links(D);
-    const int Q = D->Q, prec = D->prec;
-    const int cur = (int)(D->t & 1), nxt = cur ^ 1;
-    if (D->n_moving || D->prep_dirty || D->lists_dirty) {
-        CK(launch_fprep(D->p, D->dbodies, D->poses, D->t, D->counters + 9 + (D->t & 1), D->flags, D->chg_cnt, D->chg_cell,
-                        D->chg_val, D->chg_cap,
-                        D->apm_cnt, D->bn_cnt + 1 + nxt, nullptr, nullptr, nullptr, D->s));
-        D->prep_dirty = false;
-    }
-    if (D->lists_dirty) {
-        int rc = build_bnd_lists(D);
-        if (rc) return rc;
-    }
-    // side stream, or the main stream itself in the serial arrangement
-    cudaStream_t ss = D->side_serial ? D->s : D->s2;
-    if (!D->side_serial) {
-        CK(cudaEventRecord(D->ev_prep, D->s));
-        CK(cudaStreamWaitEvent(D->s2, D->ev_prep, 0));
-    }
-    StepBufs sb = step_bufs(D);
-    GeomArgs g = geom_args(D, true);
-    g.grid_cap = D->side_serial ? 0 : D->side_blocks;
-    if (D->n_moving) {
-        CK(launch_fgeom1(Q, D->p, g, ss));
-        CK(launch_fgeom2(Q, D->p, g, ss));
-    }
-    BndArgs ba{};
-    ba.static_cells = D->bn_static;
-    ba.static_cnt = D->bn_cnt;
-    ba.mov_cells = D->bn_mov[cur];
-    ba.mov_cnt = D->bn_cnt + 1 + cur;
-    ba.static_cap = D->bn_static_cap;
-    ba.mov_cap = D->bn_mov_cap;
-    ba.owner_t = D->owner[cur];
-    ba.owner_t1 = D->owner[nxt];
-    ba.bodies = D->dbodies;
-    ba.poses = D->poses;
-    CK(launch_bnd(Q, prec, D->p, ba, sb, D->side_serial ? D->bnd_grid_full : D->bnd_grid, ss));
-    CK(launch_finish(Q, prec, D->p, sb, ss));
-    if (D->n_free) CK(launch_free(D->p, D->dbodies, D->series, D->counters, D->counters + 9 + (D->t & 1), ss));
-    if (!D->side_serial) CK(cudaEventRecord(D->ev_side, D->s2));
-    cudaEvent_t ta = nullptr, tb = nullptr;
-    if (D->timing) {
-        int trc = timing_events(D, ta, tb);
-        if (trc) return trc;
-        CK(record_timing(D, ta));
-    }
-    CK(launch_bulk(Q, prec, D->p, sb, D->s));
-    if (D->timing) CK(record_timing(D, tb));
-    if (!D->side_serial) CK(cudaStreamWaitEvent(D->s, D->ev_side, 0));
-    D->t += 1;
-    if (D->capturing) D->cap_k += 1;
-    return LBM_OK;
-}
-
-// Link mode (reduced precision, single domain).  Stream s: prep -> cut links
-// (wall values into the solid nodes' slots, momentum exchange) -> stream-collide
-// of every fluid node (boundary nodes included; moments kept at the nodes near
-// bodies).  Side stream: after prep, the owners, covered/uncovered lists, flag
-// changes and cut links of t+1 of the moving bodies; after the cut links, the
-// end of step (series row, impulsive terms with covered nodes re-pulled from
-// fhat(t) and its wall values, refill of uncovered nodes) and the free-body
-// update.  The side stream overlaps the stream-collide pass and touches no
-// data it reads or writes: the links of t+1 go to the other list buffer, the
-// kept-moment band only gains flags, refilled nodes were solid at t.
-int do_step_links(lbm_domain *D) {
-    const int Q = D->Q, prec = D->prec;
-    const int cur = (int)(D->t & 1), nxt = cur ^ 1;
-    if (D->n_moving || D->prep_dirty || D->lists_dirty) {
-        CK(launch_fprep(D->p, D->dbodies, D->poses, D->t, D->counters + 9 + (D->t & 1), D->flags, D->chg_cnt, D->chg_cell,
-                        D->chg_val, D->chg_cap, D->apm_cnt, D->bn_cnt + 1 + nxt, D->link_cnt[cur], D->link_cnt[nxt],
-                        D->tile_pre, D->s));
-        D->prep_dirty = false;
-        D->lists_dirty = false;
-    }
-    const int scheme = step_scheme(D);
-    if (scheme != LBM_FREE_EXPLICIT) { // semi-implicit free-body schemes: one stream
-        StepBufs sb = step_bufs(D);
-        if (scheme == LBM_FREE_PREDICTOR) {
-            CK(cudaMemsetAsync(D->apm_pred_cnt, 0, sizeof(long long) * (size_t)D->nb, D->s));
-            CK(launch_fgeom1(Q, D->p, predicted_geom(D), D->s));
-        }
-        CK(launch_links(Q, prec, D->p, sb, D->links_grid, D->s));
-        cudaEvent_t ta = nullptr, tb = nullptr;
-        if (D->timing) {
-            int trc = timing_events(D, ta, tb);
-            if (trc) return trc;
-            CK(record_timing(D, ta));
-        }
-        CK(launch_bulk(Q, prec, D->p, sb, D->s));
-        if (D->timing) CK(record_timing(D, tb));
-        int rc = finish_semi(D, scheme, sb);
-        if (rc) return rc;
-        D->t += 1;
-        if (D->capturing) D->cap_k += 1;
+    int rc;
+    if (!D->nb) {
+        D->prep_dirty = D->lists_dirty = false;
+        if ((rc = bulk_pass(D, step_bufs(D)))) return rc;
+        step_done(D);
         return LBM_OK;
     }
+    if ((rc = prepare_step(D))) return rc;
+    const int scheme = step_scheme(D);
+    if (scheme != LBM_FREE_EXPLICIT) return step_semi(D, scheme);
     const bool side = !D->side_serial;
     cudaStream_t ss = side ? D->s2 : D->s;
     StepBufs sb = step_bufs(D);
@@ -800,8 +740,7 @@ int do_step_links(lbm_domain *D) {
     if (D->n_moving) {
         GeomArgs g = geom_args(D, true);
         g.grid_cap = side ? D->side_blocks : 0;
-        CK(launch_fgeom1(Q, D->p, g, ss));
-        CK(launch_fgeom2(Q, D->p, g, ss));
+        if ((rc = geometry(D, g, true, ss))) return rc;
     }
     CK(launch_links(Q, prec, D->p, sb, D->links_grid, D->s));
     if (side) {
@@ -811,17 +750,9 @@ int do_step_links(lbm_domain *D) {
     CK(launch_finish(Q, prec, D->p, sb, ss));
     if (D->n_free) CK(launch_free(D->p, D->dbodies, D->series, D->counters, D->counters + 9 + (D->t & 1), ss));
     if (side) CK(cudaEventRecord(D->ev_side, D->s2));
-    cudaEvent_t ta = nullptr, tb = nullptr;
-    if (D->timing) {
-        int trc = timing_events(D, ta, tb);
-        if (trc) return trc;
-        CK(record_timing(D, ta));
-    }
-    CK(launch_bulk(Q, prec, D->p, sb, D->s));
-    if (D->timing) CK(record_timing(D, tb));
+    if ((rc = bulk_pass(D, sb))) return rc;
     if (side) CK(cudaStreamWaitEvent(D->s, D->ev_side, 0));
-    D->t += 1;
-    if (D->capturing) D->cap_k += 1;
+    step_done(D);
     return LBM_OK;
 }
 
@@ -1187,7 +1118,7 @@ int place_bodies(lbm_domain *D, const lbm_body *hb, int n) {
     CK(launch_raster(D->Q, D->p, g, D->owner[0], 0, D->s));
     CK(cudaMemcpyAsync(D->owner[1], D->owner[0], N * sizeof(uint16_t), cudaMemcpyDeviceToDevice, D->s));
     CK(launch_flags_full(D->Q, D->p, D->owner[0], D->flags, D->s));
-    if (D->p.linkmode) CK(launch_macband(D->p, g, D->s)); // kept moments around every body
+    if (!D->batch) CK(launch_macband(D->p, g, D->s)); // kept moments around every body
     if (lists) {
         CK(launch_geom_b(D->Q, D->p, g, D->s));
         CK(launch_geom_c(D->Q, D->p, g, D->s));

@@ -122,11 +122,12 @@ __device__ void prefix_over_bodies(const Params &p, const long long *link_cnt, l
 
 // wrapped poses at t and t+1, prefixes of link counts and link tiles, and
 // the solid flags of the nodes that the previous step covered (A+) or
-// uncovered (A-), so that the flags describe the solid set of step t
+// uncovered (A-), so that the flags describe the solid set of step t (each
+// list is applied once and emptied: a body that stops moving leaves none)
 __global__ void __launch_bounds__(1024) k_prep(Params p, const BodyDev *bodies, const long long *link_cnt,
                                                long long *link_pre, long long *tile_pre, double *poses, long long t_arg,
                                                const unsigned long long *tdev, uint8_t *flags,
-                                               const long long *apm_cnt, const uint32_t *apm_cell,
+                                               long long *apm_cnt, const uint32_t *apm_cell,
                                                const int8_t *apm_sign) {
     const long long t = tdev ? (long long)*tdev : t_arg; // the device step counter, when given
     if (flags) {
@@ -139,6 +140,7 @@ __global__ void __launch_bounds__(1024) k_prep(Params p, const BodyDev *bodies, 
             }
         }
         __syncthreads();
+        for (int b = threadIdx.x; b < p.nb; b += 1024) apm_cnt[b] = 0;
     }
     prefix_over_bodies(p, link_cnt, link_pre, 0);
     prefix_over_bodies(p, link_cnt, tile_pre, 1);
@@ -197,6 +199,9 @@ __global__ void __launch_bounds__(GEOM_THREADS) k_geom_a(Params p, GeomArgs g) {
         RegionCell rc = region_cell(p, B, lo, cm.y, j);
         if (!rc.valid) continue;
         const float dist = frame_dist(p, B, F, rc);
+        // the nodes whose moments the links and refills of the next steps read
+        // (as k_fgeom1 does in link mode)
+        if (g.do_band && dist <= Rout + MAC_BAND && !(g.flags[rc.cell] & FL_MAC)) g.flags[rc.cell] |= FL_MAC;
         if (dist < Rin - 2.0f || dist > Rout + 2.0f) continue;
         const bool in_t = g.owner_t[rc.cell] == me;
         const bool in1 = inside_screened(p, B, F, rc.x, rc.y, rc.z);
@@ -701,7 +706,7 @@ cudaError_t launch_macband(const Params &p, const GeomArgs &g, cudaStream_t s) {
 
 cudaError_t launch_prep(const Params &p, const BodyDev *bodies, const long long *link_cnt, long long *link_pre,
                         long long *tile_pre, double *poses, long long t, const unsigned long long *tdev,
-                        uint8_t *flags, const long long *apm_cnt, const uint32_t *apm_cell, const int8_t *apm_sign,
+                        uint8_t *flags, long long *apm_cnt, const uint32_t *apm_cell, const int8_t *apm_sign,
                         cudaStream_t s) {
     k_prep<<<1, 1024, 0, s>>>(p, bodies, link_cnt, link_pre, tile_pre, poses, t, tdev, flags, apm_cnt, apm_cell,
                               apm_sign);

@@ -30,6 +30,7 @@ struct GeomArgs {
     long long t_link; // pose time of the links being built
     int do_apm;       // covered/uncovered lists (moving step)
     int do_flags;     // rewrite flags in the regions
+    int do_band;      // FP64 mode: set FL_MAC within R + MAC_BAND of the pose of t+1 (never cleared)
     // reduced-precision modes: flag changes for t+1, applied by the next prep
     unsigned long long *chg_cnt;
     uint32_t *chg_cell;
@@ -87,7 +88,7 @@ cudaError_t launch_finish(int Q, int prec, const Params &p, const StepBufs &sb, 
 // per step: wrapped poses at t and t+1 and the prefix of the link counts
 cudaError_t launch_prep(const Params &p, const BodyDev *bodies, const long long *link_cnt, long long *link_pre,
                         long long *tile_pre, double *poses, long long t, const unsigned long long *tdev,
-                        uint8_t *flags, const long long *apm_cnt, const uint32_t *apm_cell, const int8_t *apm_sign,
+                        uint8_t *flags, long long *apm_cnt, const uint32_t *apm_cell, const int8_t *apm_sign,
                         cudaStream_t s);
 // reduced-precision modes: poses, and the flag changes of the previous step;
 // clears the change list and the covered/uncovered counters

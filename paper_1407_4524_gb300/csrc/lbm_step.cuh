@@ -1450,9 +1450,8 @@ __device__ __forceinline__ void imp_body_exact(const Params &p, const StepBufs &
             double r[3], tq[3];
             disp(p, X, x, y, z, r);
             cross3(r, m, tq);
-            // the free-body schemes leave the solid flags to the next prep (the
-            // lists it applies are those of the displacement made)
-            if (p.free_scheme == 0) sb.flags[A] = (uint8_t)((sb.flags[A] & ~FL_SOLID) | (s > 0 ? FL_SOLID : 0));
+            // (the solid flags change in the next prep: the stream-collide pass of
+            // this step, which may still run, reads those of t)
             part[threadIdx.x][0] = m[0];
             part[threadIdx.x][1] = m[1];
             part[threadIdx.x][2] = m[2];
@@ -1579,6 +1578,37 @@ __device__ __forceinline__ void imp_body_fast(const Params &p, const StepBufs &s
     }
 }
 
+// v[0] + v[1] + ... in that order.  The chain of additions cannot be cut, so
+// the loads run ahead of it: two register tiles, one in flight while the other
+// is added (a plain loop waits for memory every four additions: 0.68 ms for
+// 9.6k links alone, 0.48 ms with the tiles, the latency of the additions).
+constexpr int SUM_TILE = 16;
+__device__ __forceinline__ double ordered_sum(const double *v, long long n) {
+    double a[SUM_TILE], b[SUM_TILE], acc = 0.0;
+    auto fetch = [&](double (&t)[SUM_TILE], long long j0) {
+#pragma unroll
+        for (int k = 0; k < SUM_TILE; ++k) t[k] = j0 + k < n ? __ldcg(v + j0 + k) : 0.0;
+    };
+    auto add = [&](const double (&t)[SUM_TILE], long long j0) {
+        if (j0 + SUM_TILE <= n) {
+#pragma unroll
+            for (int k = 0; k < SUM_TILE; ++k) acc += t[k];
+        } else {
+#pragma unroll
+            for (int k = 0; k < SUM_TILE; ++k)
+                if (j0 + k < n) acc += t[k];
+        }
+    };
+    fetch(a, 0);
+    for (long long j = 0; j < n; j += 2 * SUM_TILE) {
+        fetch(b, j + SUM_TILE);
+        add(a, j);
+        fetch(a, j + 2 * SUM_TILE);
+        add(b, j + SUM_TILE);
+    }
+    return acc;
+}
+
 // per-body sum of the link contributions into the series row of step t
 template <bool EXACT> __device__ __forceinline__ void reduce_body(const Params &p, const StepBufs &sb, int b) {
     const BodyDev &B = sb.bodies[b];
@@ -1587,9 +1617,7 @@ template <bool EXACT> __device__ __forceinline__ void reduce_body(const Params &
         const int k = threadIdx.x;
         double acc = 0.0;
         if constexpr (EXACT) { // sequential in link order (= cell, direction order of the oracle)
-            const long long cnt = sb.link_cnt[b];
-            const double *mk = sb.me + k * p.me_stride + B.link_off;
-            for (long long j = 0; j < cnt; ++j) acc += mk[j];
+            acc = ordered_sum(sb.me + k * p.me_stride + B.link_off, sb.link_cnt[b]);
         } else { // exact fixed-point sums accumulated by k_links; cleared for the next step
             unsigned long long *a = sb.acc + (long long)b * SERIES_ROW + (k < 6 ? k : k + 6);
             acc = from_fx(*a);
