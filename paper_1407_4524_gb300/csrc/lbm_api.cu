@@ -360,7 +360,7 @@ void body_params(const lbm_domain *D, const lbm_body &b, BodyDev &o) {
         o.ext[a] = e;
     }
     long long vol = (long long)o.ext[0] * o.ext[1] * o.ext[2];
-    o.nchunks = (int)((vol + GEOM_CHUNK - 1) / GEOM_CHUNK);
+    o.nchunks = (int)(((long long)o.ext[1] * o.ext[2] + GEOM_ROWS - 1) / GEOM_ROWS);
     o.link_cap = link_capacity(D, b);
     o.apm_cap = vol;
 }
@@ -739,7 +739,7 @@ int do_step(lbm_domain *D) {
     }
     if (D->n_moving) {
         GeomArgs g = geom_args(D, true);
-        g.grid_cap = side ? D->side_blocks : 0;
+        g.grid_cap = side ? 2 * D->side_blocks : 0; // (blocks of half the threads of the other kernels' cap)
         if ((rc = geometry(D, g, true, ss))) return rc;
     }
     CK(launch_links(Q, prec, D->p, sb, D->links_grid, D->s));

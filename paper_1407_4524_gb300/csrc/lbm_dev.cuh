@@ -25,9 +25,8 @@ constexpr uint8_t FL_BND = 4;   // fluid node with a solid neighbour at t (handl
 
 constexpr int SERIES_ROW = 18;  // Fs Ts Fi Ti Fm Tm
 constexpr int ME_PER_LINK = 12; // Fs Ts Fm Tm contributions of one link
-constexpr int GEOM_THREADS = 512;
-constexpr int GEOM_CELLS = 8; // consecutive region cells per thread
-constexpr int GEOM_CHUNK = GEOM_THREADS * GEOM_CELLS;
+constexpr int GEOM_THREADS = 256;
+constexpr int GEOM_ROWS = 32; // region rows (y, z) of a geometry chunk
 constexpr int REGION_MARGIN = 4;
 // link mode: moments are kept at fluid nodes within R + MAC_BAND of a body
 // (a cut link's fluid end and its x_F + c_i lie within 2 sqrt(2) of the
@@ -502,18 +501,12 @@ __device__ __forceinline__ int region_axis(int k, int lo, int len, int n, int pe
 // cos, sin of the orientation at t [18] and at t+1 [24] (15 after Xw)
 constexpr int POSE_STRIDE = 26;
 
-// region of a body covering its poses at t and t+1, dilated by `margin`
-__device__ __forceinline__ void region_lo(const Params &p, const BodyDev &b, const double *P, int margin, int lo[3]) {
-    for (int a = 0; a < 3; ++a) {
-        int n = axis_len(p, a);
-        bool full = (a == 2 && along_z(b.shape)) || b.ext[a] >= n;
-        if (full) {
-            lo[a] = 0;
-            continue;
-        }
-        double m = P[a] < P[6 + a] ? P[a] : P[6 + a];
-        lo[a] = (int)floor(m - b.R) - margin;
-    }
+// first cell along axis a of the region of a body covering its poses at t and
+// t+1, dilated by `margin`
+__device__ __forceinline__ int region_lo_axis(const Params &p, const BodyDev &b, const double *P, int margin, int a) {
+    if ((a == 2 && along_z(b.shape)) || b.ext[a] >= axis_len(p, a)) return 0;
+    const double m = P[a] < P[6 + a] ? P[a] : P[6 + a];
+    return (int)floor(m - b.R) - margin;
 }
 
 } // namespace lbm

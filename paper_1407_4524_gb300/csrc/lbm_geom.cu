@@ -4,9 +4,10 @@
 // (fluid node x_F, direction i with x_F - c_i inside the body, fractional
 // distance Delta of Sec. 2.1).
 //
-// Work is split into chunks of GEOM_THREADS consecutive cells of each body's
-// region (a box covering the body at t and t+1 plus a margin), enumerated in
-// ascending cell order even across periodic seams.  Lists are compacted with
+// Work is split into chunks of GEOM_ROWS rows of each body's region (a box
+// covering the body at t and t+1 plus a margin), cut to the shell around the
+// surface where a kernel has work and enumerated in ascending cell order even
+// across periodic seams (shell_open).  Lists are compacted with
 // block scans and per-chunk offsets, so every list is in cell order (then
 // direction order) whatever the launch configuration: the FP64 mode can then
 // sum link contributions in exactly the oracle's order.
@@ -164,130 +165,138 @@ __global__ void __launch_bounds__(1024) k_prep(Params p, const BodyDev *bodies, 
     }
 }
 
+// every kernel below: one block per chunk (or a capped grid looping over
+// them), the chunk's shell cells numbered by shell_open, GEOM_THREADS at a time
+
 __global__ void __launch_bounds__(GEOM_THREADS) k_raster(Params p, GeomArgs g, uint16_t *owner, long long) {
+    __shared__ ShellChunk c;
     const int2 cm = g.chunk_map[blockIdx.x];
     const BodyDev &B = g.bodies[cm.x];
     const double *P = g.poses + (long long)cm.x * POSE_STRIDE;
-    __shared__ Frame F;
-    if (threadIdx.x == 0) make_frame(P + 3, F);
-    __syncthreads();
-    int lo[3];
-    region_lo(p, B, P, REGION_MARGIN, lo);
-    for (int j = 0; j < GEOM_CELLS; ++j) {
-        RegionCell rc = region_cell(p, B, lo, cm.y, j);
-        if (rc.valid && inside_screened(p, B, F, rc.x, rc.y, rc.z)) owner[rc.cell] = (uint16_t)(cm.x + 1);
+    const int total = shell_open(p, B, P, 3, cm.y, -1.0f, body_rout(B) + 1.0f, c);
+    for (int e = threadIdx.x; e < total; e += GEOM_THREADS) {
+        const RegionCell rc = shell_cell(p, c, e);
+        if (inside_screened(p, B, c.F, rc.x, rc.y, rc.z)) owner[rc.cell] = (uint16_t)(cm.x + 1);
     }
 }
 
-// moving step, part a: owner at t+1 for this body's region; count A+/A-.
-// Only the shell R-2 <= |x - X(t+1)| <= R+2 can change owner (the surface
-// moves less than half a cell per step).
+// owner at t+1 of one cell of the shell R-2 .. R+2 of body b (only the shell
+// can change owner: the surface moves less than half a cell per step):
+// +1 covered, -1 uncovered, 0 neither
+__device__ __forceinline__ int update_owner(const Params &p, const GeomArgs &g, const BodyDev &B, int b, const Frame &F,
+                                            const RegionCell &rc) {
+    const uint16_t me = (uint16_t)(b + 1);
+    const bool in_t = g.owner_t[rc.cell] == me;
+    const bool in1 = inside_screened(p, B, F, rc.x, rc.y, rc.z);
+    if (in1) g.owner_t1[rc.cell] = me;
+    else if (in_t || g.owner_t1[rc.cell] == me) g.owner_t1[rc.cell] = 0;
+    return in_t == in1 ? 0 : (in1 ? 1 : -1);
+}
+
+// moving step, part a: owner at t+1 for this body's region; count A+/A-
 __global__ void __launch_bounds__(GEOM_THREADS) k_geom_a(Params p, GeomArgs g) {
+    __shared__ ShellChunk c;
     const int2 cm = g.chunk_map[blockIdx.x];
     const int b = cm.x;
     const BodyDev &B = g.bodies[b];
     const double *P = g.poses + (long long)b * POSE_STRIDE;
-    __shared__ Frame F;
-    if (threadIdx.x == 0) make_frame(P + 9, F);
-    __syncthreads();
-    int lo[3];
-    region_lo(p, B, P, REGION_MARGIN, lo);
-    const uint16_t me = (uint16_t)(b + 1);
     const float Rin = body_rin(B), Rout = body_rout(B);
-    int flags = 0;
-    for (int j = 0; j < GEOM_CELLS; ++j) {
-        RegionCell rc = region_cell(p, B, lo, cm.y, j);
-        if (!rc.valid) continue;
-        const float dist = frame_dist(p, B, F, rc);
+    const int total = shell_open(p, B, P, 9, cm.y, Rin - 2.0f, Rout + (g.do_band ? MAC_BAND : 2.0f), c);
+    int changed = 0;
+    for (int e = threadIdx.x; e < total; e += GEOM_THREADS) {
+        const RegionCell rc = shell_cell(p, c, e);
+        const float dist = frame_dist(p, B, c.F, rc);
         // the nodes whose moments the links and refills of the next steps read
         // (as k_fgeom1 does in link mode)
         if (g.do_band && dist <= Rout + MAC_BAND && !(g.flags[rc.cell] & FL_MAC)) g.flags[rc.cell] |= FL_MAC;
         if (dist < Rin - 2.0f || dist > Rout + 2.0f) continue;
-        const bool in_t = g.owner_t[rc.cell] == me;
-        const bool in1 = inside_screened(p, B, F, rc.x, rc.y, rc.z);
-        if (in1) g.owner_t1[rc.cell] = me;
-        else if (in_t || g.owner_t1[rc.cell] == me) g.owner_t1[rc.cell] = 0;
-        flags += in_t != in1;
+        changed += update_owner(p, g, B, b, c.F, rc) != 0;
     }
-    int total;
-    block_excl_scan(flags, &total);
-    if (threadIdx.x == 0) g.chunk_cnt_apm[blockIdx.x] = total;
+    int sum;
+    block_excl_scan(changed, &sum);
+    if (threadIdx.x == 0) g.chunk_cnt_apm[blockIdx.x] = sum;
+}
+
+// the cut links of cell rc to body `me`: bit i set where x - c_i is its node
+template <class L>
+__device__ __forceinline__ unsigned cut_mask(const Params &p, const uint16_t *owner, uint16_t me, const RegionCell &rc) {
+    unsigned m = 0u;
+    if (inner1(p, rc.x, rc.y, rc.z)) {
+        const long long sy = p.nx, sz = (long long)p.nx * p.ny;
+#pragma unroll
+        for (int i = 1; i < L::Q; ++i) m |= (owner[nbr1_inner<L>(rc.cell, sy, sz, i)] == me ? 1u : 0u) << i;
+    } else {
+#pragma unroll
+        for (int i = 1; i < L::Q; ++i) {
+            const long long a = nbr<L>(p, rc.x, rc.y, rc.z, i, 1);
+            m |= ((a >= 0 && owner[a] == me) ? 1u : 0u) << i;
+        }
+    }
+    return m;
 }
 
 // part b: A+/A- lists (moving step), node flags (FP64 mode), link counts
 template <class L>
 __global__ void __launch_bounds__(GEOM_THREADS) k_geom_b(Params p, GeomArgs g) {
+    __shared__ ShellChunk c;
     const int2 cm = g.chunk_map[blockIdx.x];
     const int b = cm.x;
     const BodyDev &B = g.bodies[b];
     const uint16_t me = (uint16_t)(b + 1);
     const uint16_t *owner_L = g.owner_t1; // geometry of the links being built
     const double *P = g.poses + (long long)b * POSE_STRIDE;
-    const double *XL = P + (g.t_link == g.t ? 3 : 9);
-    __shared__ Frame F;
-    if (threadIdx.x == 0) make_frame(XL, F);
-    __syncthreads();
-    int lo[3];
-    region_lo(p, B, P, REGION_MARGIN, lo);
-    const int first = blockIdx.x - cm.y; // first chunk of this body
     const float Rin = body_rin(B), Rout = body_rout(B);
-    unsigned apm_mask = 0, apm_sign = 0;
+    const int cells = shell_open(p, B, P, g.t_link == g.t ? 3 : 9, cm.y, Rin - 2.0f, Rout + (g.do_flags ? 5.5f : 2.0f), c);
+    const int first = blockIdx.x - cm.y; // first chunk of this body
+    long long at = g.do_apm ? block_sum_range(g.chunk_cnt_apm, first, cm.y) : 0;
     int nl = 0;
-    for (int j = 0; j < GEOM_CELLS; ++j) {
-        RegionCell rc = region_cell(p, B, lo, cm.y, j);
-        if (!rc.valid) continue;
-        const float dist = frame_dist(p, B, F, rc);
-        if (g.do_apm && dist >= Rin - 2.0f && dist <= Rout + 2.0f) {
-            const bool in_t = g.owner_t[rc.cell] == me, in1 = g.owner_t1[rc.cell] == me;
-            if (in_t != in1) {
-                apm_mask |= 1u << j;
-                if (in1) apm_sign |= 1u << j;
+    for (int base = 0; base < cells; base += GEOM_THREADS) {
+        const int e = base + threadIdx.x;
+        int change = 0;
+        RegionCell rc{0, 0, 0, 0};
+        if (e < cells) {
+            rc = shell_cell(p, c, e);
+            const float dist = frame_dist(p, B, c.F, rc);
+            if (g.do_apm && dist >= Rin - 2.0f && dist <= Rout + 2.0f) {
+                const bool in_t = g.owner_t[rc.cell] == me, in1 = g.owner_t1[rc.cell] == me;
+                if (in_t != in1) change = in1 ? 1 : -1;
             }
-        }
-        // node flags (FP64 mode: the moment-store flag follows the geometry of t+1;
-        // under the semi-implicit schemes a free body's pose of t+1 is known only
-        // after the step's force, so its moments are kept on the band within
-        // R + MAC_BAND of the pose the flags are built from, which holds the
-        // nodes within two links of the body at t+1 and t+2 whatever the update)
-        if (g.do_flags && dist >= Rin - 2.0f && dist <= Rout + 5.5f) {
-            uint8_t nf = node_flags<L>(p, g.owner_t, owner_L, rc.x, rc.y, rc.z, rc.cell);
-            if (p.free_scheme && B.free && dist <= Rout + MAC_BAND) nf |= FL_MAC;
-            g.flags[rc.cell] = nf;
-        }
-        if (dist >= Rin - 0.5f && dist <= Rout + 2.0f && owner_L[rc.cell] == 0) {
-#pragma unroll
-            for (int i = 1; i < L::Q; ++i) {
-                const long long a = nbr<L>(p, rc.x, rc.y, rc.z, i, 1);
-                nl += (a >= 0 ? owner_L[a] : (uint16_t)0) == me;
+            // node flags (FP64 mode, semi-implicit schemes: the moment-store flag follows the
+            // geometry of t+1; a free body's pose of t+1 is known only
+            // after the step's force, so its moments are kept on the band within
+            // R + MAC_BAND of the pose the flags are built from, which holds the
+            // nodes within two links of the body at t+1 and t+2 whatever the update)
+            if (g.do_flags && dist >= Rin - 2.0f && dist <= Rout + 5.5f) {
+                uint8_t nf = node_flags<L>(p, g.owner_t, owner_L, rc.x, rc.y, rc.z, rc.cell);
+                if (p.free_scheme && B.free && dist <= Rout + MAC_BAND) nf |= FL_MAC;
+                g.flags[rc.cell] = nf;
             }
+            if (dist >= Rin - 0.5f && dist <= Rout + 2.0f && owner_L[rc.cell] == 0)
+                nl += __popc(cut_mask<L>(p, owner_L, me, rc));
+        }
+        if (g.do_apm) {
+            int total;
+            const long long k = at + block_excl_scan(change != 0, &total);
+            if (change && k < B.apm_cap) {
+                g.apm_cell[B.apm_off + k] = (uint32_t)rc.cell;
+                g.apm_sign[B.apm_off + k] = (int8_t)change;
+            }
+            at += total;
         }
     }
-    if (g.do_apm) {
-        const long long before = block_sum_range(g.chunk_cnt_apm, first, cm.y);
-        int total;
-        long long at = before + block_excl_scan(__popc(apm_mask), &total);
-        for (int j = 0; j < GEOM_CELLS; ++j) {
-            if (!(apm_mask & (1u << j))) continue;
-            if (at < B.apm_cap) {
-                RegionCell rc = region_cell(p, B, lo, cm.y, j);
-                g.apm_cell[B.apm_off + at] = (uint32_t)rc.cell;
-                g.apm_sign[B.apm_off + at] = (int8_t)((apm_sign & (1u << j)) ? 1 : -1);
-            }
-            at++;
-        }
-        if (cm.y == B.nchunks - 1 && threadIdx.x == 0) {
-            long long n = before + total;
-            g.apm_cnt[b] = n < B.apm_cap ? n : B.apm_cap;
-        }
-    }
+    if (g.do_apm && cm.y == B.nchunks - 1 && threadIdx.x == 0) g.apm_cnt[b] = at < B.apm_cap ? at : B.apm_cap;
     int total;
     block_excl_scan(nl, &total);
     if (threadIdx.x == 0) g.chunk_cnt_link[blockIdx.x] = total;
 }
 
-// part c: fill the cut-link list of the body (cell order, then direction)
+// part c: fill the cut-link list of the body (cell order, then direction).  A
+// thread writes the directions of its cell's links; their Delta is then
+// computed one link per thread (an FP64 root costs microseconds of latency,
+// which a thread with the eight links of one cell would pay eight times)
 template <class L>
 __global__ void __launch_bounds__(GEOM_THREADS) k_geom_c(Params p, GeomArgs g) {
+    __shared__ ShellChunk c;
     const int2 cm = g.chunk_map[blockIdx.x];
     const int b = cm.x;
     const BodyDev &B = g.bodies[b];
@@ -295,58 +304,48 @@ __global__ void __launch_bounds__(GEOM_THREADS) k_geom_c(Params p, GeomArgs g) {
     const uint16_t *owner_L = g.owner_t1;
     const double *P = g.poses + (long long)b * POSE_STRIDE;
     const double *XL = P + (g.t_link == g.t ? 3 : 9);
-    __shared__ Frame F;
-    if (threadIdx.x == 0) make_frame(XL, F);
-    __syncthreads();
-    int lo[3];
-    region_lo(p, B, P, REGION_MARGIN, lo);
-    const int first = blockIdx.x - cm.y;
     const float Rin = body_rin(B), Rout = body_rout(B);
-    unsigned mask[GEOM_CELLS];
-    int nl = 0;
-#pragma unroll
-    for (int j = 0; j < GEOM_CELLS; ++j) {
-        mask[j] = 0;
-        RegionCell rc = region_cell(p, B, lo, cm.y, j);
-        if (!rc.valid) continue;
-        const float dist = frame_dist(p, B, F, rc);
-        if (dist >= Rin - 0.5f && dist <= Rout + 2.0f && owner_L[rc.cell] == 0) {
-#pragma unroll
-            for (int i = 1; i < L::Q; ++i) {
-                const long long a = nbr<L>(p, rc.x, rc.y, rc.z, i, 1);
-                if ((a >= 0 ? owner_L[a] : (uint16_t)0) == me) mask[j] |= 1u << i;
-            }
-            nl += __popc(mask[j]);
-        }
-    }
+    const int cells = shell_open(p, B, P, g.t_link == g.t ? 3 : 9, cm.y, Rin - 0.5f, Rout + 2.0f, c);
+    const int first = blockIdx.x - cm.y;
     const long long before = block_sum_range(g.chunk_cnt_link, first, cm.y);
-    int total;
-    long long at = before + block_excl_scan(nl, &total);
-#pragma unroll
-    for (int j = 0; j < GEOM_CELLS; ++j) {
-        if (!mask[j]) continue;
-        RegionCell rc = region_cell(p, B, lo, cm.y, j);
-        double d[3];
-        float df[3];
-        if (p.exact) disp(p, XL, rc.x, rc.y, rc.z, d);
-        else frame_disp_f(p, F, rc.x, rc.y, rc.z, df);
-        for (int i = 1; i < L::Q; ++i) {
-            if (!(mask[j] & (1u << i))) continue;
-            if (at < B.link_cap) {
-                const long long jj = B.link_off + at;
-                g.Lcell[jj] = (uint32_t)rc.cell;
-                g.Ldir[jj] = (uint8_t)i;
-                g.Ldelta[jj] = p.exact ? link_delta(B, d, L::cx(i), L::cy(i), L::cz(i), F.co, F.si)
-                                       : (double)link_delta_f(B.halfway, B.shape, (float)B.R, (float)B.R2, F.cof,
-                                                              F.sif, df, L::cx(i), L::cy(i), L::cz(i));
-            }
-            at++;
+    long long at = before;
+    for (int base = 0; base < cells; base += GEOM_THREADS) {
+        const int e = base + threadIdx.x;
+        unsigned m = 0u;
+        RegionCell rc{0, 0, 0, 0};
+        if (e < cells) {
+            rc = shell_cell(p, c, e);
+            const float dist = frame_dist(p, B, c.F, rc);
+            if (dist >= Rin - 0.5f && dist <= Rout + 2.0f && owner_L[rc.cell] == 0) m = cut_mask<L>(p, owner_L, me, rc);
+        }
+        int total;
+        long long k = at + block_excl_scan(__popc(m), &total);
+        for (; m; m &= m - 1, ++k) {
+            if (k >= B.link_cap) break;
+            g.Lcell[B.link_off + k] = (uint32_t)rc.cell;
+            g.Ldir[B.link_off + k] = (uint8_t)(__ffs(m) - 1);
+        }
+        at += total;
+    }
+    __syncthreads(); // the chunk's links are written
+    const long long end = at < B.link_cap ? at : B.link_cap;
+    for (long long k = before + threadIdx.x; k < end; k += GEOM_THREADS) {
+        const long long j = B.link_off + k;
+        const int i = g.Ldir[j];
+        int x, y, z;
+        coords_of(p, g.Lcell[j], x, y, z);
+        if (p.exact) {
+            double d[3];
+            disp(p, XL, x, y, z, d);
+            g.Ldelta[j] = link_delta(B, d, L::cx(i), L::cy(i), L::cz(i), c.F.co, c.F.si);
+        } else {
+            float d[3];
+            frame_disp_f(p, c.F, x, y, z, d);
+            g.Ldelta[j] = (double)link_delta_f(B.halfway, B.shape, (float)B.R, (float)B.R2, c.F.cof, c.F.sif, d, L::cx(i),
+                                               L::cy(i), L::cz(i));
         }
     }
-    if (cm.y == B.nchunks - 1 && threadIdx.x == 0) {
-        long long n = before + total;
-        g.link_cnt[b] = n < B.link_cap ? n : B.link_cap;
-    }
+    if (cm.y == B.nchunks - 1 && threadIdx.x == 0) g.link_cnt[b] = end;
 }
 
 template <class L>
@@ -441,194 +440,91 @@ __global__ void __launch_bounds__(1024) k_fprep(Params p, const BodyDev *bodies,
     }
 }
 
-// owner at t+1 in the shell R-2 <= |x - X(t+1)| <= R+2, A+/A- appended
+// owner at t+1 in the shell R-2 <= |x - X(t+1)| <= R+2, A+/A- appended; the
+// kept-moment band (link mode: the nodes whose moments the cut links of the
+// next steps read, within R + 4 of the body at t+1; never cleared)
 __global__ void __launch_bounds__(GEOM_THREADS) k_fgeom1(Params p, GeomArgs g) {
-    __shared__ Frame F;
+    __shared__ ShellChunk c;
     for (int ch = blockIdx.x; ch < g.nchunks; ch += gridDim.x) {
         const int2 cm = g.chunk_map[ch];
         const int b = cm.x;
         const BodyDev &B = g.bodies[b];
         const double *P = g.poses + (long long)b * POSE_STRIDE;
-        __syncthreads();
-        if (threadIdx.x == 0) make_frame(P + 9, F);
-        __syncthreads();
-        int lo[3];
-        region_lo(p, B, P, REGION_MARGIN, lo);
-        const uint16_t me = (uint16_t)(b + 1);
         const float Rin = body_rin(B), Rout = body_rout(B);
-        RegionWalk w;
-        walk_start(w, p, B, lo, cm.y);
-        for (int j = 0; j < GEOM_CELLS; ++j, walk_next(w)) {
-            RegionCell rc = walk_cell(w, p, lo);
-            if (!rc.valid) continue;
-            const float dist = frame_dist(p, B, F, rc);
-            // link mode: the nodes whose moments the cut links of the next
-            // steps read (within R + 4 of the body at t+1; never cleared)
-            if (p.linkmode && dist <= Rout + MAC_BAND && !(g.flags[rc.cell] & FL_MAC)) g.flags[rc.cell] |= FL_MAC;
+        const int total = shell_open(p, B, P, 9, cm.y, Rin - 2.0f, Rout + MAC_BAND, c);
+        for (int e = threadIdx.x; e < total; e += GEOM_THREADS) {
+            const RegionCell rc = shell_cell(p, c, e);
+            const float dist = frame_dist(p, B, c.F, rc);
+            if (dist <= Rout + MAC_BAND && !(g.flags[rc.cell] & FL_MAC)) g.flags[rc.cell] |= FL_MAC;
             if (dist < Rin - 2.0f || dist > Rout + 2.0f) continue;
-            const bool in_t = g.owner_t[rc.cell] == me;
-            const bool in1 = inside_screened(p, B, F, rc.x, rc.y, rc.z);
-            if (in1) g.owner_t1[rc.cell] = me;
-            else if (in_t || g.owner_t1[rc.cell] == me) g.owner_t1[rc.cell] = 0;
-            if (in_t != in1) {
+            const int change = update_owner(p, g, B, b, c.F, rc);
+            if (change) {
                 const unsigned long long at = atomicAdd((unsigned long long *)&g.apm_cnt[b], 1ull);
                 if ((long long)at < B.apm_cap) {
                     g.apm_cell[B.apm_off + at] = (uint32_t)rc.cell;
-                    g.apm_sign[B.apm_off + at] = (int8_t)(in1 ? 1 : -1);
+                    g.apm_sign[B.apm_off + at] = (int8_t)change;
                 }
             }
         }
     }
 }
 
-// flags of t+1 (solid, boundary node) in the shell R-2 .. R+3; changes appended
-template <class L>
-__global__ void __launch_bounds__(GEOM_THREADS) k_fgeom2(Params p, GeomArgs g) {
-    __shared__ Frame F;
-    for (int ch = blockIdx.x; ch < g.nchunks; ch += gridDim.x) {
-        const int2 cm = g.chunk_map[ch];
-        const int b = cm.x;
-        const BodyDev &B = g.bodies[b];
-        const double *P = g.poses + (long long)b * POSE_STRIDE;
-        __syncthreads();
-        if (threadIdx.x == 0) make_frame(P + 9, F);
-        __syncthreads();
-        int lo[3];
-        region_lo(p, B, P, REGION_MARGIN, lo);
-        const float Rin = body_rin(B), Rout = body_rout(B);
-        for (int j = 0; j < GEOM_CELLS; ++j) {
-            RegionCell rc = region_cell_i(p, B, lo, cm.y, j);
-            if (!rc.valid) continue;
-            const float dist = frame_dist(p, B, F, rc);
-            if (dist < Rin - 2.0f || dist > Rout + 3.0f) continue;
-            uint8_t nf;
-            if (g.owner_t1[rc.cell]) {
-                nf = FL_SOLID;
-            } else {
-                unsigned one = 0, lowest = 0xffffu;
-                bool mine = false;
-#pragma unroll
-                for (int i = 1; i < L::Q; ++i) {
-                    const long long a = nbr<L>(p, rc.x, rc.y, rc.z, i, 1);
-                    const unsigned o = a >= 0 ? g.owner_t1[a] : 0u;
-                    one |= o;
-                    mine |= o == (unsigned)(b + 1);
-                    if (o && o < lowest) lowest = o;
-                }
-                nf = one ? FL_BND : 0;
-                // boundary node of t+1 next to a moving body: listed by the
-                // lowest-numbered moving one (this body is moving; a
-                // lower-numbered neighbour body is looked up only if present)
-                bool list = mine && dist <= Rout + 1.5f;
-                if (list && lowest < (unsigned)(b + 1)) {
-#pragma unroll
-                    for (int i = 1; i < L::Q; ++i) {
-                        const long long a = nbr<L>(p, rc.x, rc.y, rc.z, i, 1);
-                        const unsigned o = a >= 0 ? g.owner_t1[a] : 0u;
-                        if (o && o < (unsigned)(b + 1) && g.bodies[o - 1].moving) list = false;
-                    }
-                }
-                if (list) {
-                    const unsigned long long at = atomicAdd(g.bn_mov_cnt, 1ull);
-                    if ((long long)at < g.bn_mov_cap) g.bn_mov[at] = (uint32_t)rc.cell;
-                }
-            }
-            if ((g.flags[rc.cell] & (FL_SOLID | FL_BND)) != nf) {
-                const unsigned long long at = atomicAdd(g.chg_cnt, 1ull);
-                if ((long long)at < g.chg_cap) {
-                    g.chg_cell[at] = (uint32_t)rc.cell;
-                    g.chg_val[at] = nf;
-                }
-            }
-        }
-    }
-}
-
-// link mode: the solid flags of t+1 in the shell R-2 .. R+3 (changes
-// appended; link mode reads no boundary-node flag), and the cut links of t+1
-// to this body (fluid node at t+1 within R + 1.5, direction i with x - c_i
-// inside the body at t+1, Delta in FP32 from the pose of t+1), appended to the
-// body's segment of the other list buffer: a thread first finds the links of
-// its GEOM_CELLS cells, then one block scan and one atomic per chunk place them
-// (their order does not matter: exact fixed-point sums)
+// the solid flags of t+1 in the shell R-2 .. R+3 (changes appended), and the
+// cut links of t+1 to this body (fluid node at t+1 within R + 1.5, direction i
+// with x - c_i inside the body at t+1, Delta in FP32 from the pose of t+1),
+// appended to the body's segment of the other list buffer: one block scan and
+// one atomic per tile of cells place them (their order does not matter: exact
+// fixed-point sums)
 template <class L>
 __global__ void __launch_bounds__(GEOM_THREADS) k_fgeom2l(Params p, GeomArgs g) {
-    __shared__ Frame F;
+    __shared__ ShellChunk c;
+    __shared__ unsigned long long base_s;
     for (int ch = blockIdx.x; ch < g.nchunks; ch += gridDim.x) {
         const int2 cm = g.chunk_map[ch];
         const int b = cm.x;
         const BodyDev &B = g.bodies[b];
         const double *P = g.poses + (long long)b * POSE_STRIDE;
-        __syncthreads();
-        if (threadIdx.x == 0) make_frame(P + 9, F);
-        __syncthreads();
-        int lo[3];
-        region_lo(p, B, P, REGION_MARGIN, lo);
         const float Rin = body_rin(B), Rout = body_rout(B);
         const uint16_t me = (uint16_t)(b + 1);
-        unsigned mj[GEOM_CELLS]; // directions of each cell's cut links to the body
-        int nl = 0;
-        const long long sy = p.nx, sz = (long long)p.nx * p.ny;
-        RegionWalk w;
-        walk_start(w, p, B, lo, cm.y);
-#pragma unroll
-        for (int j = 0; j < GEOM_CELLS; ++j, walk_next(w)) {
-            mj[j] = 0u;
-            const RegionCell rc = walk_cell(w, p, lo);
-            if (!rc.valid) continue;
-            const float dist = frame_dist(p, B, F, rc);
-            if (dist < Rin - 2.0f || dist > Rout + 3.0f) continue;
-            const bool solid1 = g.owner_t1[rc.cell] != 0;
-            const uint8_t nf = solid1 ? FL_SOLID : 0;
-            if ((g.flags[rc.cell] & FL_SOLID) != nf) {
-                const unsigned long long at = atomicAdd(g.chg_cnt, 1ull);
-                if ((long long)at < g.chg_cap) {
-                    g.chg_cell[at] = (uint32_t)rc.cell;
-                    g.chg_val[at] = nf;
+        const int cells = shell_open(p, B, P, 9, cm.y, Rin - 2.0f, Rout + 3.0f, c);
+        for (int tile = 0; tile < cells; tile += GEOM_THREADS) {
+            const int e = tile + threadIdx.x;
+            unsigned m = 0u; // directions of the cell's cut links to the body
+            RegionCell rc{0, 0, 0, 0};
+            if (e < cells) {
+                rc = shell_cell(p, c, e);
+                const float dist = frame_dist(p, B, c.F, rc);
+                if (dist >= Rin - 2.0f && dist <= Rout + 3.0f) {
+                    const bool solid1 = g.owner_t1[rc.cell] != 0;
+                    const uint8_t nf = solid1 ? FL_SOLID : 0;
+                    if ((g.flags[rc.cell] & FL_SOLID) != nf) {
+                        const unsigned long long at = atomicAdd(g.chg_cnt, 1ull);
+                        if ((long long)at < g.chg_cap) {
+                            g.chg_cell[at] = (uint32_t)rc.cell;
+                            g.chg_val[at] = nf;
+                        }
+                    }
+                    if (!solid1 && dist <= Rout + 1.5f) m = cut_mask<L>(p, g.owner_t1, me, rc);
                 }
             }
-            if (solid1 || dist > Rout + 1.5f) continue;
-            unsigned m = 0u;
-            if (inner1(p, rc.x, rc.y, rc.z)) {
-#pragma unroll
-                for (int i = 1; i < L::Q; ++i)
-                    m |= (g.owner_t1[nbr1_inner<L>(rc.cell, sy, sz, i)] == me ? 1u : 0u) << i;
-            } else {
-#pragma unroll
-                for (int i = 1; i < L::Q; ++i) {
-                    const long long a = nbr<L>(p, rc.x, rc.y, rc.z, i, 1);
-                    m |= ((a >= 0 && g.owner_t1[a] == me) ? 1u : 0u) << i;
+            int total;
+            const int first = block_excl_scan(__popc(m), &total); // (syncs the block)
+            if (total == 0) continue;
+            if (threadIdx.x == 0) base_s = atomicAdd((unsigned long long *)&g.link_cnt[b], (unsigned long long)total);
+            __syncthreads();
+            long long at = (long long)base_s + first;
+            if (m) {
+                float d[3];
+                frame_disp_f(p, c.F, rc.x, rc.y, rc.z, d);
+                for (; m; m &= m - 1, ++at) {
+                    if (at >= B.link_cap) break;
+                    const int i = __ffs(m) - 1;
+                    const long long j = B.link_off + at;
+                    g.Lcell[j] = (uint32_t)rc.cell;
+                    g.Ldir[j] = (uint8_t)i;
+                    g.Ldelta[j] = (double)link_delta_f(B.halfway, B.shape, (float)B.R, (float)B.R2, c.F.cof, c.F.sif, d,
+                                                       L::cx(i), L::cy(i), L::cz(i));
                 }
-            }
-            mj[j] = m;
-            nl += __popc(m);
-        }
-        int total;
-        const long long first = block_excl_scan(nl, &total); // (syncs the block)
-        __shared__ unsigned long long base_s;
-        if (threadIdx.x == 0)
-            base_s = total ? atomicAdd((unsigned long long *)&g.link_cnt[b], (unsigned long long)total) : 0ull;
-        __syncthreads();
-        long long at = (long long)base_s + first;
-        if (!nl) continue;
-        walk_start(w, p, B, lo, cm.y);
-#pragma unroll
-        for (int j = 0; j < GEOM_CELLS; ++j, walk_next(w)) {
-            const unsigned m = mj[j];
-            if (!m) continue;
-            const RegionCell rc = walk_cell(w, p, lo);
-            float df[3];
-            frame_disp_f(p, F, rc.x, rc.y, rc.z, df);
-            for (int i = 1; i < L::Q; ++i) {
-                if (!((m >> i) & 1u)) continue;
-                if (at < B.link_cap) {
-                    const long long jj = B.link_off + at;
-                    g.Lcell[jj] = (uint32_t)rc.cell;
-                    g.Ldir[jj] = (uint8_t)i;
-                    g.Ldelta[jj] = (double)link_delta_f(B.halfway, B.shape, (float)B.R, (float)B.R2, F.cof, F.sif,
-                                                        df, L::cx(i), L::cy(i), L::cz(i));
-                }
-                ++at;
             }
         }
     }
@@ -639,20 +535,16 @@ __global__ void __launch_bounds__(GEOM_THREADS) k_fgeom2l(Params p, GeomArgs g) 
 // list of step t (each node once: by the lowest-numbered neighbour body)
 template <class L>
 __global__ void __launch_bounds__(GEOM_THREADS) k_bnd_lists(Params p, GeomArgs g) {
+    __shared__ ShellChunk c;
     const int2 cm = g.chunk_map[blockIdx.x];
     const int b = cm.x;
     const BodyDev &B = g.bodies[b];
     const double *P = g.poses + (long long)b * POSE_STRIDE;
-    __shared__ Frame F;
-    if (threadIdx.x == 0) make_frame(P + 3, F);
-    __syncthreads();
-    int lo[3];
-    region_lo(p, B, P, REGION_MARGIN, lo);
     const float Rin = body_rin(B), Rout = body_rout(B);
-    for (int j = 0; j < GEOM_CELLS; ++j) {
-        RegionCell rc = region_cell(p, B, lo, cm.y, j);
-        if (!rc.valid) continue;
-        const float dist = frame_dist(p, B, F, rc);
+    const int total = shell_open(p, B, P, 3, cm.y, Rin - 0.5f, Rout + 1.5f, c);
+    for (int e = threadIdx.x; e < total; e += GEOM_THREADS) {
+        const RegionCell rc = shell_cell(p, c, e);
+        const float dist = frame_dist(p, B, c.F, rc);
         if (dist < Rin - 0.5f || dist > Rout + 1.5f || g.owner_t[rc.cell] != 0) continue;
         int minall = 1 << 20, minmov = 1 << 20;
 #pragma unroll
@@ -675,24 +567,17 @@ __global__ void __launch_bounds__(GEOM_THREADS) k_bnd_lists(Params p, GeomArgs g
     }
 }
 
-// link mode, at body placement: the nodes within R + 4 of every body at t
+// at body placement: the nodes within R + 4 of every body at t
 __global__ void __launch_bounds__(GEOM_THREADS) k_macband(Params p, GeomArgs g) {
+    __shared__ ShellChunk c;
     const int2 cm = g.chunk_map[blockIdx.x];
-    const int b = cm.x;
-    const BodyDev &B = g.bodies[b];
-    const double *P = g.poses + (long long)b * POSE_STRIDE;
-    __shared__ Frame F;
-    if (threadIdx.x == 0) make_frame(P + 3, F);
-    __syncthreads();
-    int lo[3];
-    region_lo(p, B, P, REGION_MARGIN, lo);
+    const BodyDev &B = g.bodies[cm.x];
+    const double *P = g.poses + (long long)cm.x * POSE_STRIDE;
     const float Rout = body_rout(B);
-    RegionWalk w;
-    walk_start(w, p, B, lo, cm.y);
-    for (int j = 0; j < GEOM_CELLS; ++j, walk_next(w)) {
-        RegionCell rc = walk_cell(w, p, lo);
-        if (!rc.valid) continue;
-        if (frame_dist(p, B, F, rc) <= Rout + MAC_BAND) g.flags[rc.cell] |= FL_MAC;
+    const int total = shell_open(p, B, P, 3, cm.y, -1.0f, Rout + MAC_BAND, c);
+    for (int e = threadIdx.x; e < total; e += GEOM_THREADS) {
+        const RegionCell rc = shell_cell(p, c, e);
+        if (frame_dist(p, B, c.F, rc) <= Rout + MAC_BAND) g.flags[rc.cell] |= FL_MAC;
     }
 }
 
@@ -740,14 +625,8 @@ cudaError_t launch_fgeom1(int, const Params &p, const GeomArgs &g, cudaStream_t 
 cudaError_t launch_fgeom2(int Q, const Params &p, const GeomArgs &g, cudaStream_t s) {
     if (g.nchunks == 0) return cudaSuccess;
     const int grid = g.grid_cap > 0 ? min(g.nchunks, g.grid_cap) : g.nchunks;
-    if (p.linkmode) {
-        if (Q == 9) k_fgeom2l<Lat<9>><<<grid, GEOM_THREADS, 0, s>>>(p, g);
-        else k_fgeom2l<Lat<19>><<<grid, GEOM_THREADS, 0, s>>>(p, g);
-    } else if (Q == 9) {
-        k_fgeom2<Lat<9>><<<grid, GEOM_THREADS, 0, s>>>(p, g);
-    } else {
-        k_fgeom2<Lat<19>><<<grid, GEOM_THREADS, 0, s>>>(p, g);
-    }
+    if (Q == 9) k_fgeom2l<Lat<9>><<<grid, GEOM_THREADS, 0, s>>>(p, g);
+    else k_fgeom2l<Lat<19>><<<grid, GEOM_THREADS, 0, s>>>(p, g);
     return cudaGetLastError();
 }
 

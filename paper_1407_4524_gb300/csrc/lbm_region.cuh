@@ -7,126 +7,132 @@
 namespace lbm {
 
 struct RegionCell {
-    bool valid;
     int x, y, z;
     long long cell;
 };
 
-// the j-th (0..GEOM_CELLS-1) region cell of this thread in chunk `chunk`:
-// a thread owns GEOM_CELLS consecutive cells, so per-thread counts followed
-// by a block scan keep every list in cell order
-__device__ __forceinline__ RegionCell region_cell(const Params &p, const BodyDev &B, const int lo[3], int chunk,
-                                                  int j) {
-    RegionCell rc{false, 0, 0, 0, 0};
-    const int e0 = B.ext[0], e1 = B.ext[1];
-    const int vol = e0 * e1 * B.ext[2];
-    const int k = chunk * GEOM_CHUNK + (int)threadIdx.x * GEOM_CELLS + j;
-    if (k >= vol) return rc;
-    const int kz = k / (e0 * e1);
-    const int rem = k - kz * e0 * e1;
-    const int ky = rem / e0;
-    const int kx = rem - ky * e0;
-    rc.x = region_axis(kx, lo[0], e0, p.nx, p.per[0]);
-    rc.y = region_axis(ky, lo[1], e1, p.ny, p.per[1]);
-    rc.z = region_axis(kz, lo[2], B.ext[2], p.nz, p.per[2]);
-    if (rc.x < 0 || rc.y < 0 || rc.z < 0) return rc;
-    rc.valid = true;
-    rc.cell = cell_of(p, rc.x, rc.y, rc.z);
-    return rc;
-}
-
-// the same cells as region_cell, interleaved: pass j of a chunk takes cells
-// j * GEOM_THREADS + threadIdx.x, so a warp reads consecutive cells (for the
-// kernels whose lists do not depend on the order, appended with atomics)
-__device__ __forceinline__ RegionCell region_cell_i(const Params &p, const BodyDev &B, const int lo[3], int chunk,
-                                                    int j) {
-    RegionCell rc{false, 0, 0, 0, 0};
-    const int e0 = B.ext[0], e1 = B.ext[1];
-    const int vol = e0 * e1 * B.ext[2];
-    const int k = chunk * GEOM_CHUNK + j * GEOM_THREADS + (int)threadIdx.x;
-    if (k >= vol) return rc;
-    const int kz = k / (e0 * e1);
-    const int rem = k - kz * e0 * e1;
-    const int ky = rem / e0;
-    const int kx = rem - ky * e0;
-    rc.x = region_axis(kx, lo[0], e0, p.nx, p.per[0]);
-    rc.y = region_axis(ky, lo[1], e1, p.ny, p.per[1]);
-    rc.z = region_axis(kz, lo[2], B.ext[2], p.nz, p.per[2]);
-    if (rc.x < 0 || rc.y < 0 || rc.z < 0) return rc;
-    rc.valid = true;
-    rc.cell = cell_of(p, rc.x, rc.y, rc.z);
-    return rc;
-}
-
-// The cells of region_cell_i for j = 0, 1, ... of one chunk, walked with
-// the divisions done once: the thread's first cell is split into region
-// coordinates, each step adds GEOM_THREADS cells in the same mixed radix, and
-// the periodic wrap of each axis uses the start s0 and split wr that
-// region_axis recomputes per call.
-struct RegionWalk {
-    int k, vol, kx, ky, kz, e0, e1, e2, dx, dy, dz;
-    int s0[3], wr[3], full[3];
+// The shell rlo <= |x - X| <= rhi around a body, GEOM_ROWS rows (y, z) of its
+// region at a time.  Only the shell holds work (a seventh of the region of a
+// sphere of radius 9), so a chunk's rows are cut to it first: one lane of warp
+// 0 per row takes the one or two stretches of the row that the shell covers
+// (slightly wide: the callers test each cell's distance themselves), a scan
+// numbers their cells, and every thread of the block then finds its cell e by
+// a search over the 32 row prefixes -- full warps of cells that all do the
+// work, instead of warps in which a few lanes of the box do, and blocks for
+// every 32 rows instead of every 4096 cells (a disc's whole region was one
+// block).  Bound by the latency of dependent loads and FP64 operations.
+// Measured alone, before -> after: the 135x1073 FP64 disc's geom_a + b + c
+// 169 -> 30 us, the two moving spheres of a 151x97x84 box's fgeom1 + fgeom2l
+// 89 -> 42 us.  Cells are numbered in ascending cell order, also across a
+// periodic seam.
+struct ShellChunk {
+    Frame F;
+    int lo[3], s0, split;   // region origin; its first x (wrapped) and the offset past the x seam
+    int pre[GEOM_ROWS + 1]; // cells before each row
+    int a0[GEOM_ROWS], a1[GEOM_ROWS], b0[GEOM_ROWS], b1[GEOM_ROWS]; // stretches of x offsets
+    int y[GEOM_ROWS], z[GEOM_ROWS];
 };
 
-__device__ __forceinline__ void walk_start(RegionWalk &w, const Params &p, const BodyDev &B, const int lo[3],
-                                           int chunk) {
-    w.e0 = B.ext[0];
-    w.e1 = B.ext[1];
-    w.e2 = B.ext[2];
-    w.vol = w.e0 * w.e1 * w.e2;
-    w.k = chunk * GEOM_CHUNK + (int)threadIdx.x;
-    const int plane = w.e0 * w.e1;
-    w.kz = w.k / plane;
-    const int rem = w.k - w.kz * plane;
-    w.ky = rem / w.e0;
-    w.kx = rem - w.ky * w.e0;
-    w.dz = GEOM_THREADS / plane;
-    const int r2 = GEOM_THREADS - w.dz * plane;
-    w.dy = r2 / w.e0;
-    w.dx = r2 - w.dy * w.e0;
-    const int n[3] = {p.nx, p.ny, p.nz}, len[3] = {w.e0, w.e1, w.e2};
+// Opens chunk `chunk` of body B's region for the pose P + at (at = 3: wrapped
+// pose of t, 9: of t+1); called by the whole block, syncs it; returns the
+// number of cells.
+__device__ __forceinline__ int shell_open(const Params &p, const BodyDev &B, const double *P, int at, int chunk,
+                                          float rlo, float rhi, ShellChunk &c) {
+    __syncthreads(); // the last chunk is done with
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        if (lane == 0) make_frame(P + at, c.F);
+        if (lane < 3) c.lo[lane] = region_lo_axis(p, B, P, REGION_MARGIN, lane);
+        __syncwarp();
+        const int e0 = B.ext[0], e1 = B.ext[1], rows = e1 * B.ext[2];
+        const int n = p.nx, lo = c.lo[0];
+        const bool full = p.per[0] && e0 >= n;
+        const int s0 = full || !p.per[0] ? 0 : ((lo % n) + n) % n;
+        const int split = !p.per[0] || full || s0 + e0 <= n ? e0 : n - s0;
+        const int r = chunk * GEOM_ROWS + lane;
+        const int kz = r / e1, ky = r - kz * e1;
+        int a0 = 0, a1 = 0, b0 = 0, b1 = 0;
+        int y = -1, z = -1;
+        if (r < rows) {
+            y = region_axis(ky, c.lo[1], e1, p.ny, p.per[1]);
+            z = region_axis(kz, c.lo[2], B.ext[2], p.nz, p.per[2]);
+        }
+        if (y >= 0 && z >= 0) {
+            const float dy = frame_axis(y - c.F.xi[1], c.F.fr[1], p.ny, p.per[1]);
+            const float dz = B.shape == 1 ? frame_axis(z - c.F.xi[2], c.F.fr[2], p.nz, p.per[2]) : 0.0f;
+            const float r2 = dy * dy + dz * dz, ro = rhi + 0.05f, ri = rlo - 0.05f;
+            const float h2 = ro * ro - r2, g2 = ri > 0.0f ? ri * ri - r2 : -1.0f;
+            if (full) { // the row may meet the shell across the seam: all of it
+                if (h2 >= 0.0f) a1 = n;
+            } else if (h2 >= 0.0f) {
+                const float mid = (float)(P[at - 3] - (double)lo), h = sqrtf(h2);
+                a0 = max(0, (int)ceilf(mid - h - 0.05f));
+                a1 = min(e0, (int)floorf(mid + h + 0.05f) + 1);
+                if (!p.per[0]) {
+                    a0 = max(a0, -lo);
+                    a1 = min(a1, n - lo);
+                }
+                const float g = g2 > 0.0f ? sqrtf(g2) - 0.05f : 0.0f;
+                const int end = (int)floorf(mid - g) + 1, beg = (int)ceilf(mid + g);
+                if (g > 0.0f && beg > end) { // a hole in the middle
+                    b0 = max(a0, beg);
+                    b1 = max(b0, a1);
+                    a1 = min(a1, end);
+                }
+                a1 = max(a0, a1);
+            }
+        }
+        c.y[lane] = y;
+        c.z[lane] = z;
+        c.a0[lane] = a0;
+        c.a1[lane] = a1;
+        c.b0[lane] = b0;
+        c.b1[lane] = b1;
+        const int cnt = (a1 - a0) + (b1 - b0);
+        int inc = cnt;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += v;
+        }
+        c.pre[lane] = inc - cnt;
+        if (lane == 31) c.pre[GEOM_ROWS] = inc;
+        if (lane == 0) {
+            c.s0 = s0;
+            c.split = split;
+        }
+    }
+    __syncthreads();
+    return c.pre[GEOM_ROWS];
+}
+
+// cell e (0 <= e < shell_open's count) of the open chunk
+__device__ __forceinline__ RegionCell shell_cell(const Params &p, const ShellChunk &c, int e) {
+    int r = 0;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        w.full[a] = len[a] >= n[a];
-        w.s0[a] = ((lo[a] % n[a]) + n[a]) % n[a];
-        w.wr[a] = w.s0[a] + len[a] - n[a];
+    for (int k = GEOM_ROWS / 2; k > 0; k >>= 1)
+        if (c.pre[r + k] <= e) r += k;
+    int j = e - c.pre[r];
+    const int a0 = c.a0[r], a1 = c.a1[r], b0 = c.b0[r], b1 = c.b1[r], sp = c.split;
+    // offsets past the seam come first: their wrapped x are the smaller ones
+    const int pa = max(a0, sp), pb = max(b0, sp);
+    const int na = max(0, a1 - pa), nb = max(0, b1 - pb);
+    int o;
+    if (j < na) o = pa + j;
+    else if (j < na + nb) o = pb + (j - na);
+    else {
+        j -= na + nb;
+        const int qa = max(0, min(a1, sp) - a0);
+        o = j < qa ? a0 + j : b0 + (j - qa);
     }
-}
-
-__device__ __forceinline__ void walk_next(RegionWalk &w) {
-    w.k += GEOM_THREADS;
-    w.kx += w.dx;
-    if (w.kx >= w.e0) {
-        w.kx -= w.e0;
-        ++w.ky;
+    RegionCell rc;
+    if (!p.per[0]) {
+        rc.x = c.lo[0] + o;
+    } else {
+        rc.x = c.s0 + o;
+        if (rc.x >= p.nx) rc.x -= p.nx;
     }
-    w.ky += w.dy;
-    if (w.ky >= w.e1) {
-        w.ky -= w.e1;
-        ++w.kz;
-    }
-    w.kz += w.dz;
-}
-
-// region_axis with the walk's per-axis constants
-__device__ __forceinline__ int walk_axis(const RegionWalk &w, int a, int k, int lo, int n, int periodic) {
-    if (!periodic) {
-        const int v = lo + k;
-        return (v < 0 || v >= n) ? -1 : v;
-    }
-    if (w.full[a]) return k < n ? k : -1;
-    if (w.wr[a] > 0) return k < w.wr[a] ? k : w.s0[a] + (k - w.wr[a]);
-    return w.s0[a] + k;
-}
-
-__device__ __forceinline__ RegionCell walk_cell(const RegionWalk &w, const Params &p, const int lo[3]) {
-    RegionCell rc{false, 0, 0, 0, 0};
-    if (w.k >= w.vol) return rc;
-    rc.x = walk_axis(w, 0, w.kx, lo[0], p.nx, p.per[0]);
-    rc.y = walk_axis(w, 1, w.ky, lo[1], p.ny, p.per[1]);
-    rc.z = walk_axis(w, 2, w.kz, lo[2], p.nz, p.per[2]);
-    if (rc.x < 0 || rc.y < 0 || rc.z < 0) return rc;
-    rc.valid = true;
+    rc.y = c.y[r];
+    rc.z = c.z[r];
     rc.cell = cell_of(p, rc.x, rc.y, rc.z);
     return rc;
 }
