@@ -184,6 +184,7 @@ struct lbm_domain {
     int bnd_grid = 0, bnd_grid_full = 0;
     int side_blocks = 0; // block cap of the side-stream kernels
     bool side_serial = false; // run the surface kernels before k_bulk on one stream, uncapped
+    bool tma = false;         // the stream-collide pass is the persistent kernel on bulk-copied tiles
     bool batch = false;       // a serving batch's solve: boundary-node kernel instead of link mode
     bool prep_dirty = true;
     int links_grid = 0;
@@ -595,7 +596,8 @@ int timing_events(lbm_domain *D, cudaEvent_t &a, cudaEvent_t &b) {
 // the free-body scheme a step runs (the explicit one when no body is free)
 int step_scheme(const lbm_domain *D) { return D->n_free ? D->p.free_scheme : LBM_FREE_EXPLICIT; }
 
-int geometry(lbm_domain *D, const GeomArgs &g, bool links, cudaStream_t s);
+int geometry_owners(lbm_domain *D, const GeomArgs &g, cudaStream_t s);
+int geometry_links(lbm_domain *D, const GeomArgs &g, cudaStream_t s);
 
 // semi-implicit schemes, after the stream-collide pass: the force row of step
 // t (with the impulsive terms of the previous displacement, or of the
@@ -617,7 +619,9 @@ int finish_semi(lbm_domain *D, int scheme, const StepBufs &sb) {
     const unsigned long long *tdev = D->counters + 9 + (D->t & 1);
     CK(launch_free(D->p, D->dbodies, D->series, D->counters, tdev, D->s));
     CK(launch_pose1(D->p, D->dbodies, D->poses, tdev, D->s));
-    int rc = geometry(D, geom_args(D, true), true, D->s);
+    const GeomArgs g = geom_args(D, true);
+    int rc = geometry_owners(D, g, D->s);
+    if (!rc) rc = geometry_links(D, g, D->s);
     if (rc) return rc;
     StepBufs s2 = sb;
     s2.phase = scheme == LBM_FREE_AIDUN ? PH_IMP : PH_FIX;
@@ -672,16 +676,21 @@ int prepare_step(lbm_domain *D) {
     return LBM_OK;
 }
 
-// owners, covered / uncovered lists and cut links of t+1 (moving bodies)
-int geometry(lbm_domain *D, const GeomArgs &g, bool links, cudaStream_t s) {
+// owners and covered / uncovered lists of t+1 (moving bodies)
+int geometry_owners(lbm_domain *D, const GeomArgs &g, cudaStream_t s) {
     if (D->prec == LBM_FP64) {
         CK(launch_geom_a(D->Q, D->p, g, s));
         CK(launch_geom_b(D->Q, D->p, g, s));
-        if (links) CK(launch_geom_c(D->Q, D->p, g, s));
     } else {
         CK(launch_fgeom1(D->Q, D->p, g, s));
-        if (links) CK(launch_fgeom2(D->Q, D->p, g, s));
     }
+    return LBM_OK;
+}
+
+// then its solid flags and cut links
+int geometry_links(lbm_domain *D, const GeomArgs &g, cudaStream_t s) {
+    if (D->prec == LBM_FP64) CK(launch_geom_c(D->Q, D->p, g, s));
+    else CK(launch_fgeom2(D->Q, D->p, g, s));
     return LBM_OK;
 }
 
@@ -693,10 +702,10 @@ int step_semi(lbm_domain *D, int scheme) {
         // node flags of t+1 (moments kept on a band around the free bodies) from
         // the displacement with U(t), and scheme 2's predicted lists
         const GeomArgs g = scheme == LBM_FREE_PREDICTOR ? predicted_geom(D) : geom_args(D, true);
-        if ((rc = geometry(D, g, false, D->s))) return rc;
+        if ((rc = geometry_owners(D, g, D->s))) return rc;
     } else if (scheme == LBM_FREE_PREDICTOR) {
         CK(cudaMemsetAsync(D->apm_pred_cnt, 0, sizeof(long long) * (size_t)D->nb, D->s));
-        if ((rc = geometry(D, predicted_geom(D), false, D->s))) return rc;
+        if ((rc = geometry_owners(D, predicted_geom(D), D->s))) return rc;
     }
     StepBufs sb = step_bufs(D);
     CK(launch_links(D->Q, D->prec, D->p, sb, D->links_grid, D->s));
@@ -737,16 +746,16 @@ int do_step(lbm_domain *D) {
         CK(cudaEventRecord(D->ev_prep, D->s));
         CK(cudaStreamWaitEvent(D->s2, D->ev_prep, 0));
     }
-    if (D->n_moving) {
-        GeomArgs g = geom_args(D, true);
-        g.grid_cap = side ? 2 * D->side_blocks : 0; // (blocks of half the threads of the other kernels' cap)
-        if ((rc = geometry(D, g, true, ss))) return rc;
-    }
+    GeomArgs g = geom_args(D, true);
+    g.grid_cap = side ? 2 * D->side_blocks : 0; // (blocks of half the threads of the other kernels' cap)
+    if (D->n_moving && (rc = geometry_owners(D, g, ss))) return rc;
+    if (D->n_moving && !D->tma && (rc = geometry_links(D, g, ss))) return rc;
     CK(launch_links(Q, prec, D->p, sb, D->links_grid, D->s));
     if (side) {
         CK(cudaEventRecord(D->ev_links, D->s));
         CK(cudaStreamWaitEvent(D->s2, D->ev_links, 0));
     }
+    if (D->n_moving && D->tma && (rc = geometry_links(D, g, ss))) return rc;
     CK(launch_finish(Q, prec, D->p, sb, ss));
     if (D->n_free) CK(launch_free(D->p, D->dbodies, D->series, D->counters, D->counters + 9 + (D->t & 1), ss));
     if (side) CK(cudaEventRecord(D->ev_side, D->s2));
@@ -921,8 +930,11 @@ int create_domain_impl(const lbm_domain_desc *desc, lbm_domain **out, bool batch
     int prio_lo = 0, prio_hi = 0;
     cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
     // high priority: blocks of the short side-stream kernels are dispatched
-    // as soon as bulk-kernel blocks retire, instead of after the whole grid
-    if ((e = cudaStreamCreateWithPriority(&D->s2, cudaStreamNonBlocking, prio_hi)) != cudaSuccess ||
+    // as soon as bulk-kernel blocks retire, instead of after the whole grid --
+    // except beside the persistent kernel on bulk-copied tiles, whose blocks
+    // take their SMs first and leave room for the side stream's
+    D->tma = !batch && bulk_is_tma(D->Q, D->prec, p, D->pop[0]) && bulk_is_tma(D->Q, D->prec, p, D->pop[1]);
+    if ((e = cudaStreamCreateWithPriority(&D->s2, cudaStreamNonBlocking, D->tma ? prio_lo : prio_hi)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&D->ev_prep, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&D->ev_links, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&D->ev_side, cudaEventDisableTiming)) != cudaSuccess ||

@@ -26,6 +26,7 @@ constexpr uint8_t FL_BND = 4;   // fluid node with a solid neighbour at t (handl
 constexpr int SERIES_ROW = 18;  // Fs Ts Fi Ti Fm Tm
 constexpr int ME_PER_LINK = 12; // Fs Ts Fm Tm contributions of one link
 constexpr int GEOM_THREADS = 256;
+constexpr int GEOM_MIN_BLOCKS = 5; // 48 registers in the geometry that runs beside the stream-collide pass
 constexpr int GEOM_ROWS = 32; // region rows (y, z) of a geometry chunk
 constexpr int REGION_MARGIN = 4;
 // link mode: moments are kept at fluid nodes within R + MAC_BAND of a body

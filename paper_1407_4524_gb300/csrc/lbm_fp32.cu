@@ -40,6 +40,11 @@ cudaError_t launch_finish_p12(int Q, int prec, const Params &p, const StepBufs &
     return Q == 9 ? finish_t<Lat<9>, PF16>(p, sb, s) : finish_t<Lat<19>, PF16>(p, sb, s);
 }
 
+bool bulk_is_tma(int Q, int prec, const Params &p, const void *src) {
+    if (prec != 2) return false;
+    return Q == 9 ? tma_ok<Lat<9>, PF16>(p, src) : tma_ok<Lat<19>, PF16>(p, src);
+}
+
 cudaError_t launch_bnd(int Q, int prec, const Params &p, const BndArgs &a, const StepBufs &sb, int grid,
                        cudaStream_t s) {
     if (prec == 1) return Q == 9 ? bnd_t<Lat<9>, PF32>(p, a, sb, grid, s) : bnd_t<Lat<19>, PF32>(p, a, sb, grid, s);

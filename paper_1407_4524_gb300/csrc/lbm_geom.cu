@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(1024) k_fprep(Params p, const BodyDev *bodies,
 // owner at t+1 in the shell R-2 <= |x - X(t+1)| <= R+2, A+/A- appended; the
 // kept-moment band (link mode: the nodes whose moments the cut links of the
 // next steps read, within R + 4 of the body at t+1; never cleared)
-__global__ void __launch_bounds__(GEOM_THREADS) k_fgeom1(Params p, GeomArgs g) {
+__global__ void __launch_bounds__(GEOM_THREADS, GEOM_MIN_BLOCKS) k_fgeom1(Params p, GeomArgs g) {
     __shared__ ShellChunk c;
     for (int ch = blockIdx.x; ch < g.nchunks; ch += gridDim.x) {
         const int2 cm = g.chunk_map[ch];
@@ -476,7 +476,7 @@ __global__ void __launch_bounds__(GEOM_THREADS) k_fgeom1(Params p, GeomArgs g) {
 // one atomic per tile of cells place them (their order does not matter: exact
 // fixed-point sums)
 template <class L>
-__global__ void __launch_bounds__(GEOM_THREADS) k_fgeom2l(Params p, GeomArgs g) {
+__global__ void __launch_bounds__(GEOM_THREADS, GEOM_MIN_BLOCKS) k_fgeom2l(Params p, GeomArgs g) {
     __shared__ ShellChunk c;
     __shared__ unsigned long long base_s;
     for (int ch = blockIdx.x; ch < g.nchunks; ch += gridDim.x) {

@@ -7,6 +7,7 @@
 #include "lbm_internal.h"
 #include "lbm_pair.cuh"
 #include "lbm_stage.cuh"
+#include "lbm_tma.cuh"
 
 namespace lbm {
 
@@ -73,9 +74,18 @@ template <class L, class P> cudaError_t bulk_t(const Params &p, const StepBufs &
     typename P::S *dst = (typename P::S *)sb.dst;
     const typename P::C *mt = (const typename P::C *)sb.mac_t;
     typename P::C *mt1 = (typename P::C *)sb.mac_t1;
-    bool pair = false;
+    bool pair = false, tma = false;
     if constexpr (!P::exact) pair = p.pair && pair_ok(p, fm);
-    if (pair) {
+    if constexpr (std::is_same<typename P::S, __half>::value) tma = sb.counters && tma_ok<L, P>(p, src);
+    if (tma) {
+        if constexpr (std::is_same<typename P::S, __half>::value) {
+            const bool room = sb.n_moving > 0, xf = fm == FM_XFACES;
+            const auto run = xf ? (room ? tma_launch<L, P, FM_XFACES, true> : tma_launch<L, P, FM_XFACES, false>)
+                                : (room ? tma_launch<L, P, FM_PERIODIC, true> : tma_launch<L, P, FM_PERIODIC, false>);
+            const cudaError_t e = run(p, src, dst, sb.flags, sb.counters, mt1, s);
+            if (e != cudaSuccess) return e;
+        }
+    } else if (pair) {
         if constexpr (!P::exact) k_bulk_pair<L, P><<<pair_grid(p), pair_block(p), 0, s>>>(p, src, dst, sb.flags, mt1);
     } else if (fm == FM_PERIODIC)
         k_bulk<L, P, FM_PERIODIC><<<bulk_grid(p), bulk_block(p), 0, s>>>(p, src, dst, sb.flags, mt, mt1);
