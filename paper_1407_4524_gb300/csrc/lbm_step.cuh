@@ -888,7 +888,8 @@ __global__ void __launch_bounds__(BULK_THREADS) k_load(Params p, const double *_
 // rho(x, t), u(x, t) of the cells c0 .. c0 + n - 1 from the stored fhat(x, t):
 // the collision keeps rho and adds the body force g to sum_i c_i f_i, so
 // rho_u u = sum_i c_i fhat_i - g/2 (rho_u = rho0, or rho in the standard
-// model); out[4][n], zero at solid nodes
+// model); out[4][n], zero at solid nodes.  Bound by the FP64 pipe: products
+// with 0 and 1 and the division by rho0 = 1 are left out (same results).
 template <class L, class P>
 __global__ void __launch_bounds__(BULK_THREADS) k_macros(Params p, const typename P::S *__restrict__ src,
                                                          const uint16_t *__restrict__ owner, long long c0,
@@ -898,16 +899,25 @@ __global__ void __launch_bounds__(BULK_THREADS) k_macros(Params p, const typenam
     const long long cell = c0 + k;
     double r = 0.0, j[3] = {0.0, 0.0, 0.0};
     if (owner[cell] == 0) { // fluid at t
+#pragma unroll
         for (int i = 0; i < L::Q; ++i) {
+            const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
             double v = (double)ldS(src + (long long)i * p.N + cell);
             if constexpr (!P::exact) v += L::template w<double>(i);
             r += v;
-            j[0] += (double)L::cx(i) * v;
-            j[1] += (double)L::cy(i) * v;
-            j[2] += (double)L::cz(i) * v;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                if (c[a] == 1) j[a] += v;
+                if (c[a] == -1) j[a] -= v;
+            }
         }
-        const double den = p.eq == 0 ? p.rho0 : r;
-        for (int a = 0; a < 3; ++a) j[a] = (j[a] - 0.5 * p.g[a]) / den;
+        if (!finite_x(r)) // a population is not finite: so is every component (0 * inf)
+            for (int a = 0; a < 3; ++a) j[a] += 0.0 * r;
+        for (int a = 0; a < 3; ++a) j[a] = j[a] - 0.5 * p.g[a];
+        if (p.eq != 0 || p.rho0 != 1.0) {
+            const double den = p.eq == 0 ? p.rho0 : r;
+            for (int a = 0; a < 3; ++a) j[a] = j[a] / den;
+        }
     }
     out[k] = r;
     for (int a = 0; a < 3; ++a) out[(long long)(a + 1) * n + k] = j[a];
