@@ -47,7 +47,8 @@ cudaError_t macros_t(const Params &p, const void *src, const uint16_t *owner, lo
 
 template <class L, class P> cudaError_t links_t(const Params &p, const StepBufs &sb, int grid, cudaStream_t s) {
     if (p.nb == 0 || grid <= 0) return cudaSuccess;
-    k_links<L, P><<<grid, LINK_THREADS, 0, s>>>(p, sb);
+    if (P::exact) k_links<L, P><<<grid * (LINK_THREADS / 32), 32, 0, s>>>(p, sb);
+    else k_links<L, P><<<grid, LINK_THREADS, 0, s>>>(p, sb);
     return cudaGetLastError();
 }
 

@@ -41,7 +41,7 @@
 namespace lbm {
 
 constexpr int BULK_THREADS = 128;
-constexpr int LINK_THREADS = 256;
+constexpr int LINK_THREADS = 128;
 constexpr int IMP_THREADS = 128;
 constexpr int N_COUNTERS = 16; // entries of the device counter array (StepBufs::counters)
 
@@ -1084,6 +1084,7 @@ __device__ __forceinline__ void link_work(const Params &p, const StepBufs &sb, c
     }
     // u_G = u(x_F + c_i, t) for Delta < 1/2 (Sec. 2.1)
     long long G = -1;
+    float4 mG = make_float4(0.0f, 0.0f, 0.0f, 0.0f); // (reduced modes: loaded beside the owner)
     if (delta < 0.5) {
         int g[3] = {x + cxi, y + cyi, z + czi};
         const int n[3] = {p.nx, p.ny, p.nz};
@@ -1095,7 +1096,9 @@ __device__ __forceinline__ void link_work(const Params &p, const StepBufs &sb, c
         }
         if (ok) {
             G = cell_of(p, g[0], g[1], g[2]);
-            if (sb.owner_t[G] != 0) G = -1;
+            const uint16_t solid = sb.owner_t[G];
+            if constexpr (!P::exact) mG = load_mac((const float *)sb.mac_t, G);
+            if (solid != 0) G = -1;
         }
         if (G < 0) atomicAdd(&sb.counters[0], 1ull);
     }
@@ -1146,7 +1149,6 @@ __device__ __forceinline__ void link_work(const Params &p, const StepBufs &sb, c
         const float dl = (float)delta;
         if (delta < 0.5) {
             if (G >= 0) {
-                const float4 mG = load_mac(macf, G);
                 ubf[0] = mG.y;
                 ubf[1] = mG.z;
                 ubf[2] = mG.w;
@@ -1208,18 +1210,54 @@ __device__ __forceinline__ void link_work(const Params &p, const StepBufs &sb, c
     out[11] = tm[2];
 }
 
-// wall values on cut links + per-link momentum-exchange contributions.
+// this thread's entry of the run-time table (the whole block calls it)
+template <class L> __device__ __forceinline__ void fill_tab(LatTab &tb) {
+    for (int i = threadIdx.x; i < L::Q; i += blockDim.x) {
+        tb.c[i][0] = (int8_t)L::cx(i);
+        tb.c[i][1] = (int8_t)L::cy(i);
+        tb.c[i][2] = (int8_t)L::cz(i);
+        tb.opp[i] = (int8_t)L::opp(i);
+        tb.w[i] = L::template w<double>(i);
+    }
+}
+
+// Warp sums of 12 integers a lane by halving: each exchange hands half of the
+// values left to the partner lane, 13 exchanges instead of 60.  Returns the sum
+// of component `comp` (-1: none), the same in the lanes 2k and 2k + 1.
+__device__ __forceinline__ unsigned long long warp_sum12(const unsigned long long (&v)[ME_PER_LINK], int &comp) {
+    const int lane = threadIdx.x & 31;
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
+    unsigned long long a[6], c[4], d[2];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) a[k] = (b4 ? v[k + 6] : v[k]) + __shfl_xor_sync(0xffffffffu, b4 ? v[k] : v[k + 6], 16);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) c[k] = (b3 ? a[k + 3] : a[k]) + __shfl_xor_sync(0xffffffffu, b3 ? a[k] : a[k + 3], 8);
+    c[3] = 0ull;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) d[k] = (b2 ? c[k + 2] : c[k]) + __shfl_xor_sync(0xffffffffu, b2 ? c[k] : c[k + 2], 4);
+    unsigned long long s = (b1 ? d[1] : d[0]) + __shfl_xor_sync(0xffffffffu, b1 ? d[0] : d[1], 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    const int low = 2 * (b2 ? 1 : 0) + (b1 ? 1 : 0);
+    comp = low < 3 ? 6 * (b4 ? 1 : 0) + 3 * (b3 ? 1 : 0) + low : -1;
+    return s;
+}
+
+// Wall values on cut links + per-link momentum-exchange contributions: bound by
+// the latency of the gathers (link record, x_F, owner and moments at x_F + c_i).
 // FP64 mode: one thread per link over a global index, contributions stored
-// per link and summed by k_finish in link order.  Reduced-precision modes:
-// each block iteration takes one tile of LINK_THREADS consecutive links of
-// one body and sums the tile in FP64 (fixed order), so k_finish only adds a
-// few tile partials per body.
+// per link and summed by k_finish in link order; blocks of one warp, so that
+// the links of a small body spread over the SMs' FP64 pipes (190 FP64
+// instructions a warp at 16 cycles each).  Reduced-precision modes: each block
+// iteration takes one tile of LINK_THREADS consecutive links of one body and
+// adds the tile's exact fixed-point sums.  Measured, before -> after (blocks of
+// 256 in both modes, the table filled by one thread, 60 exchanges): FP64 160
+// links 12.0 -> 9.8 us, 9.6k links 18.8 -> 12.6; FP32 500 links 6.4 -> 5.4 us.
 template <class L, class P>
 __global__ void __launch_bounds__(LINK_THREADS) k_links(Params p, StepBufs sb) {
     __shared__ LatTab tb;
-    if (threadIdx.x == 0) tb = make_tab<L>();
-    __syncthreads();
+    fill_tab<L>(tb);
     if constexpr (P::exact) {
+        __syncthreads();
         const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
         const long long gsz = (long long)gridDim.x * blockDim.x;
         const long long total = sb.link_pre[p.nb];
@@ -1269,18 +1307,18 @@ __global__ void __launch_bounds__(LINK_THREADS) k_links(Params p, StepBufs sb) {
             // the tile's sums: warp shuffles, then one atomic per block and
             // component (every tile of a body adds into the same 12 words)
             const int wid = threadIdx.x >> 5;
+            unsigned long long v[ME_PER_LINK];
 #pragma unroll
-            for (int c = 0; c < ME_PER_LINK; ++c) {
-                unsigned long long v = to_fx(outf[c]);
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-                if (lane == 0) part[wid][c] = v;
-            }
+            for (int c = 0; c < ME_PER_LINK; ++c) v[c] = to_fx(outf[c]);
+            int comp;
+            const unsigned long long sum = warp_sum12(v, comp);
+            if (comp >= 0 && !(lane & 1)) part[wid][comp] = sum;
             __syncthreads();
             if (threadIdx.x < ME_PER_LINK) {
-                unsigned long long v = 0ull;
-                for (int w = 0; w < LINK_THREADS / 32; ++w) v += part[w][threadIdx.x];
+                unsigned long long t = 0ull;
+                for (int w = 0; w < LINK_THREADS / 32; ++w) t += part[w][threadIdx.x];
                 const int c = threadIdx.x;
-                if (v) atomicAdd(sb.acc + (long long)b * SERIES_ROW + (c < 6 ? c : c + 6), v);
+                if (t) atomicAdd(sb.acc + (long long)b * SERIES_ROW + (c < 6 ? c : c + 6), t);
             }
             __syncthreads();
         }
