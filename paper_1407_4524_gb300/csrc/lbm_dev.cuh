@@ -258,18 +258,25 @@ __device__ __forceinline__ void wrap_pose(const Params &p, const double X[3], do
             continue;
         }
         double L = (double)axis_len(p, a);
-        Xw[a] = X[a] - L * floor(X[a] / L);
+        // (inside the first period floor(X / L) = 0 and Xw = X: the chain of an
+        // FP64 division, microseconds of latency, is left to the others)
+        Xw[a] = (X[a] >= 0.0 && X[a] <= 0.999 * L) ? X[a] : X[a] - L * floor(X[a] / L);
     }
 }
 
 // minimum-image displacement along one axis from the unwrapped pose X
 // (reading of the torque reference, Eq. H of Sec. 3): v = x - X, then on a
 // periodic axis v - L floor(v / L + 1/2) -- the oracle's expression, each
-// operation rounded explicitly so that no unit's contraction flags change it
+// operation rounded explicitly so that no unit's contraction flags change it.
 __device__ __forceinline__ double axis_disp(const Params &p, int a, double x, double X) {
     const double v = __dsub_rn(x, X);
     if (!p.per[a]) return v;
     const double L = (double)axis_len(p, a);
+    // (well inside half a period floor(v / L + 1/2) = 0 and the image is v itself:
+    // no division -- every link and covered node of a body that has not crossed
+    // a seam: the 512x256 moving cylinders' step 32.5 -> 28 us, the 151x97x84
+    // moving spheres' 92 -> 86 us)
+    if (fabs(v) <= 0.499 * L) return v;
     return __dsub_rn(v, __dmul_rn(L, floor(__dadd_rn(__ddiv_rn(v, L), 0.5))));
 }
 
