@@ -364,7 +364,8 @@ void body_params(const lbm_domain *D, const lbm_body &b, BodyDev &o) {
         o.ext[a] = e;
     }
     long long vol = (long long)o.ext[0] * o.ext[1] * o.ext[2];
-    o.nchunks = (int)(((long long)o.ext[1] * o.ext[2] + GEOM_ROWS - 1) / GEOM_ROWS);
+    const int rows = geom_rows(D->p.nz);
+    o.nchunks = (int)(((long long)o.ext[1] * o.ext[2] + rows - 1) / rows);
     o.link_cap = link_capacity(D, b);
     o.apm_cap = vol;
 }

@@ -27,7 +27,11 @@ constexpr int SERIES_ROW = 18;  // Fs Ts Fi Ti Fm Tm
 constexpr int ME_PER_LINK = 12; // Fs Ts Fm Tm contributions of one link
 constexpr int GEOM_THREADS = 256;
 constexpr int GEOM_MIN_BLOCKS = 5; // 48 registers in the geometry that runs beside the stream-collide pass
-constexpr int GEOM_ROWS = 32; // region rows (y, z) of a geometry chunk
+constexpr int GEOM_ROWS = 32; // region rows (y, z) of a geometry chunk at most
+// A plane's body has few rows with long stretches (a disc of radius 12: 33 rows,
+// 700 shell cells): eight of them make one pass of a block; a ball has a
+// thousand short ones.
+__host__ __device__ inline int geom_rows(int nz) { return nz == 1 ? 8 : GEOM_ROWS; }
 constexpr int REGION_MARGIN = 4;
 // link mode: moments are kept at fluid nodes within R + MAC_BAND of a body
 // (a cut link's fluid end and its x_F + c_i lie within 2 sqrt(2) of the

@@ -4,7 +4,7 @@
 // (fluid node x_F, direction i with x_F - c_i inside the body, fractional
 // distance Delta of Sec. 2.1).
 //
-// Work is split into chunks of GEOM_ROWS rows of each body's region (a box
+// Work is split into chunks of geom_rows rows of each body's region (a box
 // covering the body at t and t+1 plus a margin), cut to the shell around the
 // surface where a kernel has work and enumerated in ascending cell order even
 // across periodic seams (shell_open).  Lists are compacted with
@@ -474,11 +474,13 @@ __global__ void __launch_bounds__(GEOM_THREADS, GEOM_MIN_BLOCKS) k_fgeom1(Params
 // with x - c_i inside the body at t+1, Delta in FP32 from the pose of t+1),
 // appended to the body's segment of the other list buffer: one block scan and
 // one atomic per tile of cells place them (their order does not matter: exact
-// fixed-point sums)
+// fixed-point sums), then each thread takes one link (few cells have links, and
+// those have up to nine)
 template <class L>
 __global__ void __launch_bounds__(GEOM_THREADS, GEOM_MIN_BLOCKS) k_fgeom2l(Params p, GeomArgs g) {
     __shared__ ShellChunk c;
     __shared__ unsigned long long base_s;
+    __shared__ uint16_t list[GEOM_THREADS * (L::Q - 1)]; // (cell of the tile, direction)
     for (int ch = blockIdx.x; ch < g.nchunks; ch += gridDim.x) {
         const int2 cm = g.chunk_map[ch];
         const int b = cm.x;
@@ -508,24 +510,26 @@ __global__ void __launch_bounds__(GEOM_THREADS, GEOM_MIN_BLOCKS) k_fgeom2l(Param
                 }
             }
             int total;
-            const int first = block_excl_scan(__popc(m), &total); // (syncs the block)
+            int at = block_excl_scan(__popc(m), &total); // (syncs the block)
             if (total == 0) continue;
             if (threadIdx.x == 0) base_s = atomicAdd((unsigned long long *)&g.link_cnt[b], (unsigned long long)total);
+            for (; m; m &= m - 1, ++at) list[at] = (uint16_t)(threadIdx.x * 32 + (__ffs(m) - 1));
             __syncthreads();
-            long long at = (long long)base_s + first;
-            if (m) {
+            // the tile's links, one a thread
+            for (int l = threadIdx.x; l < total; l += GEOM_THREADS) {
+                const long long k = (long long)base_s + l;
+                if (k >= B.link_cap) break;
+                const int i = list[l] & 31;
+                const RegionCell q = shell_cell(p, c, tile + (list[l] >> 5));
                 float d[3];
-                frame_disp_f(p, c.F, rc.x, rc.y, rc.z, d);
-                for (; m; m &= m - 1, ++at) {
-                    if (at >= B.link_cap) break;
-                    const int i = __ffs(m) - 1;
-                    const long long j = B.link_off + at;
-                    g.Lcell[j] = (uint32_t)rc.cell;
-                    g.Ldir[j] = (uint8_t)i;
-                    g.Ldelta[j] = (double)link_delta_f(B.halfway, B.shape, (float)B.R, (float)B.R2, c.F.cof, c.F.sif, d,
-                                                       L::cx(i), L::cy(i), L::cz(i));
-                }
+                frame_disp_f(p, c.F, q.x, q.y, q.z, d);
+                const long long j = B.link_off + k;
+                g.Lcell[j] = (uint32_t)q.cell;
+                g.Ldir[j] = (uint8_t)i;
+                g.Ldelta[j] = (double)link_delta_f(B.halfway, B.shape, (float)B.R, (float)B.R2, c.F.cof, c.F.sif, d,
+                                                   L::cx(i), L::cy(i), L::cz(i));
             }
+            __syncthreads(); // the next tile writes the list
         }
     }
 }

@@ -11,7 +11,7 @@ struct RegionCell {
     long long cell;
 };
 
-// The shell rlo <= |x - X| <= rhi around a body, GEOM_ROWS rows (y, z) of its
+// The shell rlo <= |x - X| <= rhi around a body, geom_rows rows (y, z) of its
 // region at a time.  Only the shell holds work (a seventh of the region of a
 // sphere of radius 9), so a chunk's rows are cut to it first: one lane of warp
 // 0 per row takes the one or two stretches of the row that the shell covers
@@ -22,8 +22,8 @@ struct RegionCell {
 // every 32 rows instead of every 4096 cells (a disc's whole region was one
 // block).  Bound by the latency of dependent loads and FP64 operations.
 // Measured alone, before -> after: the 135x1073 FP64 disc's geom_a + b + c
-// 169 -> 30 us, the two moving spheres of a 151x97x84 box's fgeom1 + fgeom2l
-// 89 -> 42 us.  Cells are numbered in ascending cell order, also across a
+// 169 -> 22 us, the two moving spheres of a 151x97x84 box's fgeom1 + fgeom2l
+// 89 -> 31 us, two cylinders' 26 -> 14 us.  Cells are numbered in ascending cell order, also across a
 // periodic seam.
 struct ShellChunk {
     Frame F;
@@ -49,7 +49,8 @@ __device__ __forceinline__ int shell_open(const Params &p, const BodyDev &B, con
         const bool full = p.per[0] && e0 >= n;
         const int s0 = full || !p.per[0] ? 0 : ((lo % n) + n) % n;
         const int split = !p.per[0] || full || s0 + e0 <= n ? e0 : n - s0;
-        const int r = chunk * GEOM_ROWS + lane;
+        const int rpc = geom_rows(p.nz);
+        const int r = lane < rpc ? chunk * rpc + lane : rows;
         const int kz = r / e1, ky = r - kz * e1;
         int a0 = 0, a1 = 0, b0 = 0, b1 = 0;
         int y = -1, z = -1;
