@@ -38,6 +38,8 @@ cudaError_t launch_init_p0(int Q, const Params &p, void *dst, void *mac, const u
 cudaError_t launch_links_p0(int Q, const Params &p, const StepBufs &sb, int grid, cudaStream_t s);
 cudaError_t launch_bulk_p0(int Q, const Params &p, const StepBufs &sb, cudaStream_t s);
 cudaError_t launch_finish_p0(int Q, const Params &p, const StepBufs &sb, cudaStream_t s);
+cudaError_t launch_zouhe_p0(int Q, const Params &p, const StepBufs &sb, cudaStream_t s);
+cudaError_t launch_zouhe_p12(int Q, int prec, const Params &p, const StepBufs &sb, cudaStream_t s);
 cudaError_t launch_init_p12(int Q, int prec, const Params &p, void *dst, void *mac, const uint8_t *flags,
                             const double u0[3], cudaStream_t s);
 cudaError_t launch_links_p12(int Q, int prec, const Params &p, const StepBufs &sb, int grid, cudaStream_t s);
@@ -72,6 +74,9 @@ cudaError_t launch_links(int Q, int prec, const Params &p, const StepBufs &sb, i
 }
 cudaError_t launch_bulk(int Q, int prec, const Params &p, const StepBufs &sb, cudaStream_t s) {
     return prec == 0 ? launch_bulk_p0(Q, p, sb, s) : launch_bulk_p12(Q, prec, p, sb, s);
+}
+cudaError_t launch_zouhe(int Q, int prec, const Params &p, const StepBufs &sb, cudaStream_t s) {
+    return prec == 0 ? launch_zouhe_p0(Q, p, sb, s) : launch_zouhe_p12(Q, prec, p, sb, s);
 }
 cudaError_t launch_finish(int Q, int prec, const Params &p, const StepBufs &sb, cudaStream_t s) {
     return prec == 0 ? launch_finish_p0(Q, p, sb, s) : launch_finish_p12(Q, prec, p, sb, s);
@@ -194,8 +199,8 @@ struct lbm_domain {
     int64_t t = 0;
     // side stream: in the reduced-precision modes the geometry of t+1 and the
     // end-of-step kernel run on it, concurrently with the bulk kernel
-    cudaStream_t s2 = nullptr;
-    cudaEvent_t ev_prep = nullptr, ev_links = nullptr, ev_side = nullptr;
+    cudaStream_t s2 = nullptr, s3 = nullptr;
+    cudaEvent_t ev_prep = nullptr, ev_links = nullptr, ev_side = nullptr, ev_own = nullptr, ev_third = nullptr;
     // timing of the bulk kernel
     bool timing = false;
     std::vector<cudaEvent_t> ev;
@@ -714,6 +719,7 @@ int step_semi(lbm_domain *D, int scheme) {
     StepBufs sb = step_bufs(D);
     CK(launch_links(D->Q, D->prec, D->p, sb, D->links_grid, D->s));
     if ((rc = bulk_pass(D, sb))) return rc;
+    CK(launch_zouhe(D->Q, D->prec, D->p, sb, D->s));
     if ((rc = finish_semi(D, scheme, sb))) return rc;
     step_done(D);
     return LBM_OK;
@@ -721,22 +727,28 @@ int step_semi(lbm_domain *D, int scheme) {
 
 // One step.  Stream s: prep -> cut links (wall values into the solid nodes'
 // slots, momentum exchange) -> stream-collide of every fluid node (moments
-// kept at the nodes near bodies).  Side stream: after prep, the owners,
-// covered / uncovered lists and cut links of t+1 of the moving bodies; after
-// the cut links, the end of step (series row, impulsive terms with covered
-// nodes re-pulled from fhat(t) and its wall values, refill of uncovered nodes)
-// and the free-body update.  The side stream overlaps the stream-collide pass
-// and touches no data it reads or writes: the links of t+1 go to the other
-// list buffer, the kept-moment band only gains flags, solid flags change in
-// the next prep, refilled nodes were solid at t.  In FP64 mode this hides the
-// sequential link sums (0.68 ms for the 9.6k links of the 256x128x128 sphere
-// channel, whose stream-collide pass takes 1.80 ms: step 2.49 -> 1.84 ms).
+// kept at the nodes near bodies).  Second stream: after prep, the owners and
+// covered / uncovered lists of t+1 of the moving bodies; after the cut links,
+// the end of step (series row, impulsive terms with covered nodes re-pulled
+// from fhat(t) and its wall values, refill of uncovered nodes) and the
+// free-body update.  Third stream: the Zou-He face nodes (after the cut links;
+// the pass skips them), the solid flags and cut links of t+1 (after the
+// owners; they need nothing of the end of step, nor it of them).  Both overlap
+// the stream-collide pass and touch no data it reads or writes: the links of
+// t+1 go to the other list buffer, the kept-moment band only gains flags,
+// solid flags change in the next prep, refilled nodes were solid at t, the
+// free-body update writes no field of a body's record that the geometry reads.
+// In FP64 mode this hides the sequential link sums (0.68 ms for the 9.6k links
+// of the 256x128x128 sphere channel, whose stream-collide pass takes 1.80 ms:
+// step 2.49 -> 1.84 ms).
 int do_step(lbm_domain *D) {
     const int Q = D->Q, prec = D->prec;
     int rc;
     if (!D->nb) {
         D->prep_dirty = D->lists_dirty = false;
-        if ((rc = bulk_pass(D, step_bufs(D)))) return rc;
+        const StepBufs sb = step_bufs(D);
+        if ((rc = bulk_pass(D, sb))) return rc;
+        CK(launch_zouhe(Q, prec, D->p, sb, D->s));
         step_done(D);
         return LBM_OK;
     }
@@ -744,27 +756,35 @@ int do_step(lbm_domain *D) {
     const int scheme = step_scheme(D);
     if (scheme != LBM_FREE_EXPLICIT) return step_semi(D, scheme);
     const bool side = !D->side_serial;
-    cudaStream_t ss = side ? D->s2 : D->s;
+    // (no third stream beside the persistent pass: there is room for one block
+    // of the side kernels an SM, the 512x256x256 FP16 swarm's pass of 602 steps
+    // took 289 ms with two streams, 305 with three)
+    const bool third = side && !D->tma && (D->n_moving || D->p.zouhe);
+    cudaStream_t s2 = side ? D->s2 : D->s, s3 = third ? D->s3 : s2;
+    auto wait = [&](cudaStream_t on, cudaEvent_t ev, cudaStream_t of) { // `on` waits for what `of` has been given so far
+        if (!side) return cudaSuccess;
+        const cudaError_t e = cudaEventRecord(ev, of);
+        return e == cudaSuccess ? cudaStreamWaitEvent(on, ev, 0) : e;
+    };
     StepBufs sb = step_bufs(D);
-    if (side) {
-        CK(cudaEventRecord(D->ev_prep, D->s));
-        CK(cudaStreamWaitEvent(D->s2, D->ev_prep, 0));
-    }
     GeomArgs g = geom_args(D, true);
     g.grid_cap = side ? 2 * D->side_blocks : 0; // (blocks of half the threads of the other kernels' cap)
-    if (D->n_moving && (rc = geometry_owners(D, g, ss))) return rc;
-    if (D->n_moving && !D->tma && (rc = geometry_links(D, g, ss))) return rc;
-    CK(launch_links(Q, prec, D->p, sb, D->links_grid, D->s));
-    if (side) {
-        CK(cudaEventRecord(D->ev_links, D->s));
-        CK(cudaStreamWaitEvent(D->s2, D->ev_links, 0));
+    CK(wait(s2, D->ev_prep, D->s));
+    if (D->n_moving) {
+        if ((rc = geometry_owners(D, g, s2))) return rc;
+        if (third) CK(wait(s3, D->ev_own, s2));
+        if (!D->tma && !D->p.zouhe && (rc = geometry_links(D, g, s3))) return rc;
     }
-    if (D->n_moving && D->tma && (rc = geometry_links(D, g, ss))) return rc;
-    CK(launch_finish(Q, prec, D->p, sb, ss));
-    if (D->n_free) CK(launch_free(D->p, D->dbodies, D->series, D->counters, D->counters + 9 + (D->t & 1), ss));
-    if (side) CK(cudaEventRecord(D->ev_side, D->s2));
+    CK(launch_links(Q, prec, D->p, sb, D->links_grid, D->s));
+    CK(wait(s2, D->ev_links, D->s));
+    if (third && D->p.zouhe) CK(cudaStreamWaitEvent(s3, D->ev_links, 0));
+    CK(launch_zouhe(Q, prec, D->p, sb, s3));
+    if (D->n_moving && (D->tma || D->p.zouhe) && (rc = geometry_links(D, g, s3))) return rc;
+    CK(launch_finish(Q, prec, D->p, sb, s2));
+    if (D->n_free) CK(launch_free(D->p, D->dbodies, D->series, D->counters, D->counters + 9 + (D->t & 1), s2));
     if ((rc = bulk_pass(D, sb))) return rc;
-    if (side) CK(cudaStreamWaitEvent(D->s, D->ev_side, 0));
+    CK(wait(D->s, D->ev_side, s2));
+    if (third) CK(wait(D->s, D->ev_third, s3));
     step_done(D);
     return LBM_OK;
 }
@@ -939,7 +959,10 @@ int create_domain_impl(const lbm_domain_desc *desc, lbm_domain **out, bool batch
     // take their SMs first and leave room for the side stream's
     D->tma = !batch && bulk_is_tma(D->Q, D->prec, p, D->pop[0]) && bulk_is_tma(D->Q, D->prec, p, D->pop[1]);
     if ((e = cudaStreamCreateWithPriority(&D->s2, cudaStreamNonBlocking, D->tma ? prio_lo : prio_hi)) != cudaSuccess ||
+        (e = cudaStreamCreateWithPriority(&D->s3, cudaStreamNonBlocking, D->tma ? prio_lo : prio_hi)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&D->ev_prep, cudaEventDisableTiming)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&D->ev_own, cudaEventDisableTiming)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&D->ev_third, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&D->ev_links, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&D->ev_side, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaStreamCreateWithFlags(&D->sio, cudaStreamNonBlocking)) != cudaSuccess ||
@@ -978,6 +1001,12 @@ int lbm_destroy_domain(lbm_domain *D) {
         cudaStreamSynchronize(D->s2);
         cudaStreamDestroy(D->s2);
     }
+    if (D->s3) {
+        cudaStreamSynchronize(D->s3);
+        cudaStreamDestroy(D->s3);
+    }
+    if (D->ev_own) cudaEventDestroy(D->ev_own);
+    if (D->ev_third) cudaEventDestroy(D->ev_third);
     if (D->ev_prep) cudaEventDestroy(D->ev_prep);
     if (D->ev_links) cudaEventDestroy(D->ev_links);
     if (D->ev_side) cudaEventDestroy(D->ev_side);

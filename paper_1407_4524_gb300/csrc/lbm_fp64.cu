@@ -24,6 +24,9 @@ cudaError_t launch_links_p0(int Q, const Params &p, const StepBufs &sb, int grid
 cudaError_t launch_bulk_p0(int Q, const Params &p, const StepBufs &sb, cudaStream_t s) {
     return Q == 9 ? bulk_t<Lat<9>, PF64>(p, sb, s) : bulk_t<Lat<19>, PF64>(p, sb, s);
 }
+cudaError_t launch_zouhe_p0(int Q, const Params &p, const StepBufs &sb, cudaStream_t s) {
+    return Q == 9 ? zouhe_t<Lat<9>, PF64>(p, sb, s) : zouhe_t<Lat<19>, PF64>(p, sb, s);
+}
 cudaError_t launch_finish_p0(int Q, const Params &p, const StepBufs &sb, cudaStream_t s) {
     return Q == 9 ? finish_t<Lat<9>, PF64>(p, sb, s) : finish_t<Lat<19>, PF64>(p, sb, s);
 }

@@ -83,6 +83,7 @@ cudaError_t launch_init(int Q, int prec, const Params &p, void *dst, void *mac, 
                         const double u0[3], cudaStream_t s);
 cudaError_t launch_links(int Q, int prec, const Params &p, const StepBufs &sb, int grid, cudaStream_t s);
 cudaError_t launch_bulk(int Q, int prec, const Params &p, const StepBufs &sb, cudaStream_t s);
+cudaError_t launch_zouhe(int Q, int prec, const Params &p, const StepBufs &sb, cudaStream_t s);
 // whether launch_bulk takes the kernel on bulk-copied tiles (one persistent
 // block an SM) for this domain
 bool bulk_is_tma(int Q, int prec, const Params &p, const void *src);

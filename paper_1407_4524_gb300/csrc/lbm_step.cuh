@@ -42,6 +42,7 @@ namespace lbm {
 
 constexpr int BULK_THREADS = 128;
 constexpr int LINK_THREADS = 128;
+constexpr int ZOUHE_THREADS = 32; // few face nodes with long chains: one warp a block spreads them over the SMs
 constexpr int IMP_THREADS = 128;
 constexpr int N_COUNTERS = 16; // entries of the device counter array (StepBufs::counters)
 
@@ -985,7 +986,7 @@ __global__ void __launch_bounds__(BULK_THREADS, P::exact ? 4 : bulk_min_blocks<F
 // y-lo, y-hi, z-lo, z-hi); a node on several Zou-He faces is taken by the
 // first of them.
 template <class L, class P>
-__global__ void __launch_bounds__(BULK_THREADS) k_zouhe(Params p, const typename P::S *__restrict__ src,
+__global__ void __launch_bounds__(ZOUHE_THREADS) k_zouhe(Params p, const typename P::S *__restrict__ src,
                                                         typename P::S *__restrict__ dst,
                                                         const uint8_t *__restrict__ flags,
                                                         const typename P::C *__restrict__ mac_t,
