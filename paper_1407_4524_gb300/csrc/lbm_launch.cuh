@@ -11,10 +11,24 @@
 
 namespace lbm {
 
+// Threads of a row's blocks.  Rows of up to BULK_THREADS nodes: the warps the
+// row has (a block holds the registers of idle warps until it ends: the 93x61x57
+// duct's step 16.5 -> 15.2 us with 96 threads instead of 128).  Longer rows: in
+// FP64 mode, with 16 warps an SM, the size that leaves the fewest idle warps,
+// the larger of two that leave as many (135x1073 disc 75 -> 69 us with 96); in
+// the reduced modes BULK_THREADS (151x97x84: 66.2 us, 67.5 with 96).
 inline dim3 bulk_block(const Params &p) {
-    int bx = BULK_THREADS;
-    while (bx > 32 && bx / 2 >= p.nx) bx /= 2;
-    return dim3(bx, 1, 1);
+    if (p.nx <= BULK_THREADS) return dim3((p.nx + 31) / 32 * 32, 1, 1);
+    if (!p.exact) return dim3(BULK_THREADS, 1, 1);
+    int best = BULK_THREADS, least = 0;
+    for (int bx = BULK_THREADS; bx >= 64; bx -= 32) {
+        const int threads = (p.nx + bx - 1) / bx * bx;
+        if (least == 0 || threads < least) {
+            best = bx;
+            least = threads;
+        }
+    }
+    return dim3(best, 1, 1);
 }
 
 inline dim3 bulk_grid(const Params &p) {

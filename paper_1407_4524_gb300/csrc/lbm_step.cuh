@@ -506,6 +506,7 @@ __device__ __forceinline__ void face_terms(const Params &p, const typename P::S 
             f[i] = f[i] + 2.0 * L::template w<double>(i) * rhow * 3.0 * cuB;
         }
     } else {
+        if (!inlet_only) return; // walls at rest: the bounced population as it is
         float rhow = p.rho0f;
         if (p.eq != 0) {
             float dr, uu[3];
@@ -514,10 +515,10 @@ __device__ __forceinline__ void face_terms(const Params &p, const typename P::S 
         }
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) {
-            if (!((bounce >> i) & 1u)) continue;
-            const double uB0 = ((inlet_only >> i) & 1u) ? inlet_u(p, y, L::cy(i)) : 0.0;
-            const float cuB = (float)L::cx(i) * (float)uB0;
-            f[i] = fmaf(6.0f * L::template w<float>(i) * rhow, cuB, (float)f[i]);
+            if (!((bounce >> i) & 1u) || L::cx(i) == 0) continue; // (no u_B along c_i)
+            float uB0 = 0.0f;
+            if ((inlet_only >> i) & 1u) uB0 = p.inlet_parabolic ? (float)inlet_u(p, y, L::cy(i)) : p.u_inf;
+            f[i] = fmaf(6.0f * L::template w<float>(i) * rhow, (float)L::cx(i) * uB0, (float)f[i]);
         }
     }
 }
