@@ -915,6 +915,7 @@ int create_domain_impl(const lbm_domain_desc *desc, lbm_domain **out, bool batch
         p.gravity[k] = d.gravity[k];
     }
     p.omegaf = (float)p.omega;
+    p.tauf = (float)p.tau;
     p.rho0f = (float)d.rho0;
     p.inv_rho0f = 1.0f / p.rho0f;
     p.keepf = 1.0f - p.omegaf;
@@ -2159,6 +2160,7 @@ int lbm_batch_admit(lbm_batch *B, const lbm_domain_desc *desc, const lbm_body *h
         // poses of t = 0 and the boundary-node list (all static)
         cudaError_t e = launch_fprep(D->p, D->dbodies, D->poses, 0, nullptr, D->flags, D->chg_cnt, D->chg_cell, D->chg_val,
                                      D->chg_cap, D->apm_cnt, D->bn_cnt + 2, nullptr, nullptr, nullptr, D->s);
+        if (e == cudaSuccess) e = launch_body_f32(D->p, D->dbodies, D->poses, D->s);
         if (e == cudaSuccess && (rc = build_bnd_lists(D))) {
             lbm_destroy_domain(D);
             return rc;

@@ -58,21 +58,13 @@ __global__ void __launch_bounds__(BND_THREADS) k_bbnd(const SolveDev *__restrict
         const SolveDev &sv = solves[slots[k_slot]];
         if (!sv.active) continue;
         const int cur = (int)(sv.t & 1);
-        BndArgs a{};
-        a.static_cells = sv.bn_static;
-        a.static_cnt = sv.bn_cnt;
-        a.static_cap = sv.bn_cap;
-        a.owner_t = sv.owner;
-        a.owner_t1 = sv.owner;
-        a.bodies = sv.bodies;
-        a.poses = sv.poses;
         StepBufs sb{};
         sb.src = sv.pop[cur];
         sb.dst = sv.pop[cur ^ 1];
         sb.counters = sv.counters;
         sb.acc = sv.acc;
         unsigned nl = 0;
-        bnd_node<L, P>(sv.p, a, sb, sv.bn_static[k - node_pre[k_slot]], true, nl);
+        bnd_node<L, P>(sv.p, sv.bodies, sv.owner, sb, sv.bn_static[k - node_pre[k_slot]], nl);
         if (lane == 0 && nl) atomicAdd(&sv.counters[3], (unsigned long long)nl);
     }
 }

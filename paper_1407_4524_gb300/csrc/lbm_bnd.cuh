@@ -1,22 +1,20 @@
-// lbm_bnd.cuh -- boundary-node kernel of the reduced-precision modes.
+// lbm_bnd.cuh -- boundary nodes of served solves (reduced precision, static
+// bodies).
 //
 // A boundary node is a fluid node with at least one solid neighbour at t:
-// the node x_F = x_A + c_i of a cut link (Sec. 2.1).  k_bulk skips these nodes
-// (flag FL_BND); this kernel runs on the side stream beside k_bulk and does
-// their whole step.  One warp per node, one lane per lattice direction i:
+// the node x_F = x_A + c_i of a cut link (Sec. 2.1).  The stream-collide pass
+// of a served solve skips these nodes (flag FL_BND); k_bbnd runs beside it and
+// does their whole step.  One warp per node, one lane per lattice direction i:
 //   lane i pulls fhat_i(x - c_i, t) (Eq. streaming) or, if x - c_i is solid,
 //   evaluates the wall value of Eq. Fillipova_interpolation (Delta from the
 //   body pose, u_bf and chi of Sec. 2.1, u_G from the moments of fhat at
 //   x + c_i) and the link's momentum-exchange terms (Eqs. flow_force_2,
 //   flow_torque_2, ForceInMovementMovingFrame, TorqueInMovementMovingFrame),
 //   summed exactly in fixed point per body;
-// moments are warp reductions; the node is collided and stored.  A node that
-// a body covers at t+1 keeps its streamed f(x, t+1) for the impulsive terms
-// of k_finish.
-//
-// Node lists: nodes whose solid neighbours all belong to static bodies are
-// listed once; nodes next to a moving body are listed per step by k_fgeom2
-// (a node next to several moving bodies is listed by the lowest-numbered one).
+// moments are warp reductions; the node is collided and stored.  The bodies'
+// records are read in FP32 (BodyDev::flf ..): converting the FP64 ones cost 30
+// instructions a node on the FP64 pipe (16 cycles each, one pipe an SM): the
+// nodes of eight spheres 40.8 -> 35.4 us.
 #pragma once
 
 #include "lbm_internal.h"
@@ -33,8 +31,8 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 // the step of boundary node `cell` (one warp; lane = lattice direction)
 template <class L, class P>
-__device__ __forceinline__ void bnd_node(const Params &p, const BndArgs &a, const StepBufs &sb, long long cell,
-                                         bool from_static, unsigned &nlinks) {
+__device__ __forceinline__ void bnd_node(const Params &p, const BodyDev *bodies, const uint16_t *owner,
+                                         const StepBufs &sb, long long cell, unsigned &nlinks) {
     using S = typename P::S;
     const int lane = threadIdx.x & 31;
     const bool act = lane < L::Q;
@@ -50,18 +48,14 @@ __device__ __forceinline__ void bnd_node(const Params &p, const BndArgs &a, cons
     const long long sc = i == 0 ? cell : nbr<L>(p, x, y, z, i, 1);      // pull source x - c_i
     const long long G = act && i > 0 ? nbr<L>(p, x, y, z, ib, 1) : -1; // x + c_i
     // every load that depends on the node alone is issued here, together:
-    // the owners at t (node, pull sources, x + c_i) and t+1, fhat(x, t) and
-    // the pulled fhat_i(x - c_i, t) (not used where x - c_i is solid)
-    const uint16_t own = a.owner_t[cell], own1 = a.owner_t1[cell];
-    const uint16_t o = (act && i > 0 && sc >= 0) ? a.owner_t[sc] : (uint16_t)0;
-    const uint16_t oG = G >= 0 ? a.owner_t[G] : (uint16_t)1;
+    // the owners (node, pull sources, x + c_i), fhat(x, t) and the pulled
+    // fhat_i(x - c_i, t) (not used where x - c_i is solid)
+    const uint16_t own = owner[cell];
+    const uint16_t o = (act && i > 0 && sc >= 0) ? owner[sc] : (uint16_t)0;
+    const uint16_t oG = G >= 0 ? owner[G] : (uint16_t)1;
     const float fo = act ? ldP(src + (long long)i * N + cell) : 0.0f;
     const float fp = (act && sc >= 0) ? ldS(src + (long long)i * N + sc) : 0.0f;
     if (own != 0) return; // warp-uniform
-    if (from_static) { // a moving body next to it: that body's list has it
-        const bool mv = o != 0 && a.bodies[o - 1].moving;
-        if (__any_sync(0xffffffffu, mv)) return;
-    }
     const unsigned cutmask = __ballot_sync(0xffffffffu, o != 0);
     if (!cutmask) return;
     // moments of the collided populations fhat(x, t) (= those of f(x, t))
@@ -90,26 +84,22 @@ __device__ __forceinline__ void bnd_node(const Params &p, const BndArgs &a, cons
     for (int c = 0; c < ME_PER_LINK; ++c) v[c] = 0.0f;
     const int bi = (int)o - 1;
     if (o) {
-        const BodyDev &Bi = a.bodies[bi];
-        const double *Pf = a.poses + (long long)bi * POSE_STRIDE + 12; // floor, frac of the pose at t
+        const BodyDev &Bi = bodies[bi];
         float d[3];
         const int c3[3] = {x, y, z};
-        for (int q = 0; q < 3; ++q) d[q] = frame_axis(c3[q] - (int)Pf[q], (float)Pf[3 + q], axis_len(p, q), p.per[q]);
-        const double *Po = a.poses + (long long)bi * POSE_STRIDE + 18; // orientation at t
-        const float dl = link_delta_f(Bi.halfway, Bi.shape, (float)Bi.R, (float)Bi.R2, (float)Po[0], (float)Po[1],
-                                      d, cxi, cyi, czi);
+        for (int q = 0; q < 3; ++q) d[q] = frame_axis(c3[q] - Bi.flf[q], Bi.frf[q], axis_len(p, q), p.per[q]);
+        const float dl = link_delta_f(Bi.halfway, Bi.shape, Bi.Rf, Bi.R2f, Bi.cof, Bi.sif, d, cxi, cyi, czi);
         const float rb[3] = {d[0] - dl * cxi, d[1] - dl * cyi, d[2] - dl * czi};
-        const float W0 = (float)Bi.W[0], W1 = (float)Bi.W[1], W2 = (float)Bi.W[2];
-        const float uB[3] = {(float)Bi.U[0] + (W1 * rb[2] - W2 * rb[1]),
-                             (float)Bi.U[1] + (W2 * rb[0] - W0 * rb[2]),
-                             (float)Bi.U[2] + (W0 * rb[1] - W1 * rb[0])};
+        const float W0 = Bi.Wf[0], W1 = Bi.Wf[1], W2 = Bi.Wf[2];
+        const float uB[3] = {Bi.Uf[0] + (W1 * rb[2] - W2 * rb[1]), Bi.Uf[1] + (W2 * rb[0] - W0 * rb[2]),
+                             Bi.Uf[2] + (W0 * rb[1] - W1 * rb[0])};
         float ubf[3], chi;
         if (dl < 0.5f) {
             // u_bf = u_G = u(x_F + c_i, t), chi = (2 Delta - 1)/(tau - 2)
             if (G >= 0 && oG == 0) { // x + c_i fluid at t
                 float drG;
                 moments_hat<L>(p, src, G, drG, ubf);
-                chi = (2.0f * dl - 1.0f) / ((float)p.tau - 2.0f);
+                chi = (2.0f * dl - 1.0f) / (p.tauf - 2.0f);
             } else {
                 ubf[0] = uF[0];
                 ubf[1] = uF[1];
@@ -121,7 +111,7 @@ __device__ __forceinline__ void bnd_node(const Params &p, const BndArgs &a, cons
             // u_bf = u_F + 3/(2 Delta) (u_B - u_F), chi = (2 Delta - 1)/(tau + 1/2)
             const float k3 = 3.0f / (2.0f * dl);
             for (int q = 0; q < 3; ++q) ubf[q] = fmaf(k3, uB[q] - uF[q], uF[q]);
-            chi = (2.0f * dl - 1.0f) / ((float)p.tau + 0.5f);
+            chi = (2.0f * dl - 1.0f) / (p.tauf + 0.5f);
         }
         // fictitious equilibrium g_ib (Eq. Fillipova_equilibrium), deviation form
         const float cbu = -(cxi * ubf[0] + cyi * ubf[1] + czi * ubf[2]);
@@ -151,9 +141,8 @@ __device__ __forceinline__ void bnd_node(const Params &p, const BndArgs &a, cons
     } else if (act) {
         fi = sc >= 0 ? fp : pull_edge<L, P>(p, src, (const float *)nullptr, x, y, z, cell, i);
     }
-    // collision (or the streamed values of a node covered at t+1)
-    float out = fi;
-    if (own1 == 0) {
+    float out; // collision
+    {
         const float dr = warp_sum(fi);
         float j0 = warp_sum(cxi * fi), j1 = warp_sum(cyi * fi), j2 = warp_sum(czi * fi);
         if (p.has_force) {
@@ -204,29 +193,6 @@ __device__ __forceinline__ void bnd_node(const Params &p, const BndArgs &a, cons
         unsigned long long *acc = sb.acc + (long long)bi * SERIES_ROW;
         for (int c = 0; c < ME_PER_LINK; ++c) atomicAdd(acc + (c < 6 ? c : c + 6), to_fx(v[c]));
     }
-}
-
-template <class L, class P>
-__global__ void __launch_bounds__(BND_THREADS) k_bnd(Params p, BndArgs a, StepBufs sb) {
-    const int lane = threadIdx.x & 31;
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const long long ns = (long long)min((unsigned long long)a.static_cap, *a.static_cnt);
-    const long long nm = (long long)min((unsigned long long)a.mov_cap, *a.mov_cnt);
-    unsigned nlinks = 0;
-    for (long long k = warp; k < ns + nm; k += nwarps) {
-        const bool from_static = k < ns;
-        const long long cell = from_static ? a.static_cells[k] : a.mov_cells[k - ns];
-        bnd_node<L, P>(p, a, sb, cell, from_static, nlinks);
-    }
-    if (lane == 0 && nlinks) atomicAdd(&sb.counters[3], (unsigned long long)nlinks);
-}
-
-template <class L, class P>
-cudaError_t bnd_t(const Params &p, const BndArgs &a, const StepBufs &sb, int grid, cudaStream_t s) {
-    if (grid <= 0) return cudaSuccess;
-    k_bnd<L, P><<<grid, BND_THREADS, 0, s>>>(p, a, sb);
-    return cudaGetLastError();
 }
 
 } // namespace lbm

@@ -162,7 +162,7 @@ struct Params {
     double tau, omega, rho0, u_in;
     double g[3];
     double gravity[3]; // acceleration of the free bodies
-    float omegaf, rho0f, u_inf;
+    float omegaf, rho0f, u_inf, tauf;
     float inv_rho0f;  // 1 / rho0f (correctly rounded, as the device division)
     float keepf;      // 1 - omegaf
     float gf[3];
@@ -184,6 +184,10 @@ struct BodyDev {
     double density_ratio;         // free bodies: body density / rho0
     double R2;                    // ellipse: second semi-axis (R is the first, R >= R2)
     double theta0;                // ellipse: orientation about z at step t0
+    // FP32 record of a served solve's body (static; written at its admission):
+    // pose floor and fraction, orientation, radii, velocities
+    int flf[3];
+    float frf[3], cof, sif, Rf, R2f, Uf[3], Wf[3];
 };
 
 // shape codes: 0 cylinder (x-y disc, along z), 1 sphere, 2 ellipse (x-y, along z)

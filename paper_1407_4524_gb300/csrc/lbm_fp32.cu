@@ -1,7 +1,6 @@
 // lbm_fp32.cu -- reduced-precision modes: FP32 arithmetic with populations
 // stored as deviations f - w in FP32 (p1) or FP16 (p2).
 #include "lbm_launch.cuh"
-#include "lbm_bnd.cuh"
 
 namespace lbm {
 
@@ -47,12 +46,6 @@ cudaError_t launch_finish_p12(int Q, int prec, const Params &p, const StepBufs &
 bool bulk_is_tma(int Q, int prec, const Params &p, const void *src) {
     if (prec != 2) return false;
     return Q == 9 ? tma_ok<Lat<9>, PF16>(p, src) : tma_ok<Lat<19>, PF16>(p, src);
-}
-
-cudaError_t launch_bnd(int Q, int prec, const Params &p, const BndArgs &a, const StepBufs &sb, int grid,
-                       cudaStream_t s) {
-    if (prec == 1) return Q == 9 ? bnd_t<Lat<9>, PF32>(p, a, sb, grid, s) : bnd_t<Lat<19>, PF32>(p, a, sb, grid, s);
-    return Q == 9 ? bnd_t<Lat<9>, PF16>(p, a, sb, grid, s) : bnd_t<Lat<19>, PF16>(p, a, sb, grid, s);
 }
 
 } // namespace lbm

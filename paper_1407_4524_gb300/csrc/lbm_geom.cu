@@ -613,6 +613,31 @@ cudaError_t launch_fprep(const Params &p, const BodyDev *bodies, double *poses, 
 }
 
 
+namespace {
+__global__ void k_body_f32(Params p, BodyDev *bodies, const double *poses) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= p.nb) return;
+    BodyDev &B = bodies[b];
+    const double *P = poses + (long long)b * POSE_STRIDE;
+    for (int a = 0; a < 3; ++a) {
+        B.flf[a] = (int)P[12 + a];
+        B.frf[a] = (float)P[15 + a];
+        B.Uf[a] = (float)B.U[a];
+        B.Wf[a] = (float)B.W[a];
+    }
+    B.cof = (float)P[18];
+    B.sif = (float)P[19];
+    B.Rf = (float)B.R;
+    B.R2f = (float)B.R2;
+}
+} // namespace
+
+cudaError_t launch_body_f32(const Params &p, BodyDev *bodies, const double *poses, cudaStream_t s) {
+    if (p.nb == 0) return cudaSuccess;
+    k_body_f32<<<(p.nb + 63) / 64, 64, 0, s>>>(p, bodies, poses);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_bnd_lists(int Q, const Params &p, const GeomArgs &g, cudaStream_t s) {
     if (g.nchunks == 0) return cudaSuccess;
     if (Q == 9) k_bnd_lists<Lat<9>><<<g.nchunks, GEOM_THREADS, 0, s>>>(p, g);

@@ -46,18 +46,6 @@ struct GeomArgs {
     int grid_cap; // > 0: at most this many blocks (side-stream kernels)
 };
 
-// arguments of the boundary-node kernel (reduced-precision modes)
-struct BndArgs {
-    const uint32_t *static_cells;
-    const unsigned long long *static_cnt;
-    const uint32_t *mov_cells; // nodes of step t next to moving bodies
-    const unsigned long long *mov_cnt;
-    long long static_cap, mov_cap;
-    const uint16_t *owner_t, *owner_t1;
-    const BodyDev *bodies;
-    const double *poses;
-};
-
 // One resident solve of a serving batch (reduced-precision modes, static
 // bodies): everything the batched kernels need to step it.
 struct SolveDev {
@@ -103,6 +91,8 @@ cudaError_t launch_fprep(const Params &p, const BodyDev *bodies, double *poses, 
                          const uint32_t *chg_cell, const uint8_t *chg_val, long long chg_cap, long long *apm_cnt,
                          unsigned long long *bn_mov_next_cnt, const long long *link_cnt_t, long long *link_cnt_t1,
                          long long *tile_pre, cudaStream_t s);
+// served solves: the FP32 record of each (static) body
+cudaError_t launch_body_f32(const Params &p, BodyDev *bodies, const double *poses, cudaStream_t s);
 // link mode: FL_MAC on the nodes within R + MAC_BAND of every body at t
 cudaError_t launch_macband(const Params &p, const GeomArgs &g, cudaStream_t s);
 
@@ -116,10 +106,6 @@ cudaError_t launch_flags_full(int Q, const Params &p, const uint16_t *owner, uin
 // reduced-precision modes: owner(t+1) + unordered A+/A- lists; flag changes
 cudaError_t launch_fgeom1(int Q, const Params &p, const GeomArgs &g, cudaStream_t s);
 cudaError_t launch_fgeom2(int Q, const Params &p, const GeomArgs &g, cudaStream_t s);
-// reduced-precision modes: boundary nodes of every body (pull, wall values,
-// momentum exchange, collision) -- runs beside k_bulk
-cudaError_t launch_bnd(int Q, int prec, const Params &p, const BndArgs &a, const StepBufs &sb, int grid,
-                       cudaStream_t s);
 // batched serving kernels: one tick = bulk (per group), boundary nodes (per
 // group), finish (every solve).  A group is a lattice, a storage type
 // (BK_FP32 / BK_FP16) and a face mode; a bulk work item (slot, row, x0, 0)

@@ -378,15 +378,15 @@ __device__ __forceinline__ void collide_f(const Params &p, float f[], float drho
     }
 }
 
-__device__ __forceinline__ float dgeq_f(const Params &p, const LatTab &tb, int ib, float drhoF, const float ubf[3],
-                                        const float uF[3]) {
+__device__ __forceinline__ float dgeq_f(const Params &p, const LatTab &tb, const float *wf, int ib, float drhoF,
+                                        const float ubf[3], const float uF[3]) {
     float c0 = tb.c[ib][0], c1 = tb.c[ib][1], c2 = tb.c[ib][2];
     float cbu = c0 * ubf[0] + c1 * ubf[1] + c2 * ubf[2];
     float cbF = c0 * uF[0] + c1 * uF[1] + c2 * uF[2];
     float uFsq = uF[0] * uF[0] + uF[1] * uF[1] + uF[2] * uF[2];
     float poly = 3.0f * cbu + 4.5f * cbF * cbF - 1.5f * uFsq;
     float rr = p.eq == 0 ? p.rho0f : 1.0f + drhoF;
-    return (float)tb.w[ib] * fmaf(rr, poly, drhoF);
+    return wf[ib] * fmaf(rr, poly, drhoF);
 }
 
 // ========================================================= fixed point ==
@@ -1040,15 +1040,26 @@ __global__ void __launch_bounds__(ZOUHE_THREADS) k_zouhe(Params p, const typenam
 // flow_torque_2), moving-frame force and torque (Eqs.
 // ForceInMovementMovingFrame / TorqueInMovementMovingFrame); by Eq.
 // Equalities they need exactly the wall value and fhat_ib(x_F, t).
+
+// node of x_G = x_F + c_i, -1 outside a non-periodic face
+__device__ __forceinline__ long long link_g(const Params &p, int x, int y, int z, int cxi, int cyi, int czi) {
+    int g[3] = {x + cxi, y + cyi, z + czi};
+    const int n[3] = {p.nx, p.ny, p.nz};
+    bool ok = true;
+    for (int a = 0; a < 3; ++a) {
+        if (g[a] >= 0 && g[a] < n[a]) continue;
+        if (!p.per[a]) ok = false;
+        else g[a] += g[a] < 0 ? n[a] : -n[a];
+    }
+    return ok ? cell_of(p, g[0], g[1], g[2]) : -1;
+}
+
+// FP64 mode
 template <class L, class P>
-__device__ __forceinline__ void link_work(const Params &p, const StepBufs &sb, const LatTab &tb,
-                                          const BodyDev &B, const double *X, long long j, double out[ME_PER_LINK],
-                                          float outf[ME_PER_LINK]) {
-    using S = typename P::S;
-    using C = typename P::C;
-    S *pop = (S *)sb.src;
-    const C *mac = (const C *)sb.mac_t;
-    (void)mac;
+__device__ __forceinline__ void link_exact(const Params &p, const StepBufs &sb, const LatTab &tb, const BodyDev &B,
+                                           const double *X, long long j, double out[ME_PER_LINK]) {
+    double *pop = (double *)sb.src;
+    const double *mac = (const double *)sb.mac_t;
     const long long N = p.N;
     const long long cell = sb.Lcell[j];
     const int i = sb.Ldir[j];
@@ -1059,157 +1070,167 @@ __device__ __forceinline__ void link_work(const Params &p, const StepBufs &sb, c
     const int ib = tb.opp[i];
     const long long A =
         cell_of(p, wrap_axis(x - cxi, p.nx), wrap_axis(y - cyi, p.ny), wrap_axis(z - czi, p.nz));
-    double d[3], uB[3];
-    if constexpr (P::exact) {
-        double rB[3];
-        disp(p, X, x, y, z, d);
-        rB[0] = d[0] - delta * cxi;
-        rB[1] = d[1] - delta * cyi;
-        rB[2] = d[2] - delta * czi;
-        body_velocity(B, rB, uB);
-    } else { // FP32 link geometry (reduced-precision modes)
-        const double *Pf = X + 9; // floor(Xw), frac(Xw)
-        const int c3[3] = {x, y, z};
-        float df[3], rb[3];
-        for (int a = 0; a < 3; ++a) df[a] = frame_axis(c3[a] - (int)Pf[a], (float)Pf[3 + a], axis_len(p, a), p.per[a]);
-        const float dl = (float)delta;
-        rb[0] = df[0] - dl * cxi;
-        rb[1] = df[1] - dl * cyi;
-        rb[2] = df[2] - dl * czi;
-        const float W0 = (float)B.W[0], W1 = (float)B.W[1], W2 = (float)B.W[2];
-        uB[0] = (float)B.U[0] + (W1 * rb[2] - W2 * rb[1]);
-        uB[1] = (float)B.U[1] + (W2 * rb[0] - W0 * rb[2]);
-        uB[2] = (float)B.U[2] + (W0 * rb[1] - W1 * rb[0]);
-        d[0] = df[0];
-        d[1] = df[1];
-        d[2] = df[2];
-    }
+    double d[3], uB[3], rB[3];
+    disp(p, X, x, y, z, d);
+    rB[0] = d[0] - delta * cxi;
+    rB[1] = d[1] - delta * cyi;
+    rB[2] = d[2] - delta * czi;
+    body_velocity(B, rB, uB);
     // u_G = u(x_F + c_i, t) for Delta < 1/2 (Sec. 2.1)
     long long G = -1;
-    float4 mG = make_float4(0.0f, 0.0f, 0.0f, 0.0f); // (reduced modes: loaded beside the owner)
     if (delta < 0.5) {
-        int g[3] = {x + cxi, y + cyi, z + czi};
-        const int n[3] = {p.nx, p.ny, p.nz};
-        bool ok = true;
-        for (int a = 0; a < 3; ++a) {
-            if (g[a] >= 0 && g[a] < n[a]) continue;
-            if (!p.per[a]) ok = false;
-            else g[a] += g[a] < 0 ? n[a] : -n[a];
+        G = link_g(p, x, y, z, cxi, cyi, czi);
+        if (G >= 0 && sb.owner_t[G] != 0) G = -1;
+        if (G < 0) atomicAdd(&sb.counters[0], 1ull);
+    }
+    const double fb = ldP(pop + (long long)ib * N + cell);
+    const double rhoF = mac[4 * cell];
+    const double uF[3] = {mac[4 * cell + 1], mac[4 * cell + 2], mac[4 * cell + 3]};
+    double ubf[3], chi;
+    if (delta < 0.5) {
+        if (G >= 0) {
+            for (int a = 0; a < 3; ++a) ubf[a] = mac[4 * G + 1 + a];
+            chi = (2.0 * delta - 1.0) / (p.tau - 2.0);
+        } else {
+            for (int a = 0; a < 3; ++a) ubf[a] = uF[a];
+            chi = 0.0;
         }
-        if (ok) {
-            G = cell_of(p, g[0], g[1], g[2]);
+    } else {
+        double k3 = 3.0 / (2.0 * delta);
+        for (int a = 0; a < 3; ++a) ubf[a] = uF[a] + k3 * (uB[a] - uF[a]);
+        chi = (2.0 * delta - 1.0) / (p.tau + 0.5);
+    }
+    double g = geq_x(p, tb, ib, rhoF, ubf, uF);
+    double rhow = p.eq == 0 ? p.rho0 : rhoF;
+    double cuB = (double)cxi * uB[0] + (double)cyi * uB[1] + (double)czi * uB[2];
+    double bc = (1.0 - chi) * fb + chi * g + 2.0 * tb.w[i] * rhow * 3.0 * cuB;
+    stS(pop + (long long)i * N + A, bc);
+    const double fa = bc;
+    double sum = fa + fb, ps[3], pm[3], ts[3], tm[3];
+    ps[0] = -cxi * sum;
+    ps[1] = -cyi * sum;
+    ps[2] = -czi * sum;
+    const int cb[3] = {-cxi, -cyi, -czi};
+    const int cc[3] = {cxi, cyi, czi};
+    for (int a = 0; a < 3; ++a) pm[a] = -(cc[a] - uB[a]) * fa + (cb[a] - uB[a]) * fb;
+    cross3(d, ps, ts);
+    cross3(d, pm, tm);
+    for (int a = 0; a < 3; ++a) {
+        out[a] = ps[a];
+        out[3 + a] = ts[a];
+        out[6 + a] = pm[a];
+        out[9 + a] = tm[a];
+    }
+}
+
+// what the links of one body share, in FP32 (reduced-precision modes): floor
+// and fraction of the pose of t, velocities.  Filled by twelve threads of a
+// block, a value each: a conversion from FP64 a link and value took the FP64
+// pipe (2 lanes a clock) longer than the gathers take (64 spheres' links 27.5
+// -> 22 us).
+struct LinkBody {
+    int fl[3];
+    float fr[3], U[3], W[3];
+};
+__device__ __forceinline__ void fill_link_body(LinkBody &lb, const BodyDev &B, const double *X) {
+    const int t = threadIdx.x;
+    const double *Pf = X + 9; // floor(Xw), frac(Xw)
+    if (t < 3) lb.fl[t] = (int)Pf[t];
+    else if (t < 6) lb.fr[t - 3] = (float)Pf[t];
+    else if (t < 9) lb.U[t - 6] = (float)B.U[t - 6];
+    else if (t < 12) lb.W[t - 9] = (float)B.W[t - 9];
+}
+
+// reduced-precision modes (wf: the weights in FP32)
+template <class L, class P>
+__device__ __forceinline__ void link_fast(const Params &p, const StepBufs &sb, const LatTab &tb, const float *wf,
+                                          const LinkBody &lb, long long j, float out[ME_PER_LINK]) {
+    using S = typename P::S;
+    S *pop = (S *)sb.src;
+    const float *mac = (const float *)sb.mac_t;
+    const long long N = p.N;
+    const long long cell = sb.Lcell[j];
+    const int i = sb.Ldir[j];
+    const float dl = (float)sb.Ldelta[j];
+    int x, y, z;
+    coords_of(p, cell, x, y, z);
+    const int cxi = tb.c[i][0], cyi = tb.c[i][1], czi = tb.c[i][2];
+    const int ib = tb.opp[i];
+    const float fb = ldP(pop + (long long)ib * N + cell);
+    // moments of f(t) at x_F (and at x_F + c_i): kept by the previous
+    // stream-collide pass (or the refill, or the initial state)
+    const float4 mF = load_mac(mac, cell);
+    // u_G = u(x_F + c_i, t) for Delta < 1/2 (Sec. 2.1)
+    long long G = -1;
+    float4 mG = make_float4(0.0f, 0.0f, 0.0f, 0.0f); // (loaded beside the owner)
+    if (dl < 0.5f) {
+        G = link_g(p, x, y, z, cxi, cyi, czi);
+        if (G >= 0) {
             const uint16_t solid = sb.owner_t[G];
-            if constexpr (!P::exact) mG = load_mac((const float *)sb.mac_t, G);
+            mG = load_mac(mac, G);
             if (solid != 0) G = -1;
         }
         if (G < 0) atomicAdd(&sb.counters[0], 1ull);
     }
-    double fa, fb, ps[3], pm[3];
-    if constexpr (P::exact) {
-        fb = ldP(pop + (long long)ib * N + cell);
-        const double rhoF = mac[4 * cell];
-        const double uF[3] = {mac[4 * cell + 1], mac[4 * cell + 2], mac[4 * cell + 3]};
-        double ubf[3], chi;
-        if (delta < 0.5) {
-            if (G >= 0) {
-                for (int a = 0; a < 3; ++a) ubf[a] = mac[4 * G + 1 + a];
-                chi = (2.0 * delta - 1.0) / (p.tau - 2.0);
-            } else {
-                for (int a = 0; a < 3; ++a) ubf[a] = uF[a];
-                chi = 0.0;
-            }
+    const long long A =
+        cell_of(p, wrap_axis(x - cxi, p.nx), wrap_axis(y - cyi, p.ny), wrap_axis(z - czi, p.nz));
+    const int c3[3] = {x, y, z};
+    float d[3], rb[3], uB[3];
+    for (int a = 0; a < 3; ++a) d[a] = frame_axis(c3[a] - lb.fl[a], lb.fr[a], axis_len(p, a), p.per[a]);
+    rb[0] = d[0] - dl * cxi;
+    rb[1] = d[1] - dl * cyi;
+    rb[2] = d[2] - dl * czi;
+    const float W0 = lb.W[0], W1 = lb.W[1], W2 = lb.W[2];
+    uB[0] = lb.U[0] + (W1 * rb[2] - W2 * rb[1]);
+    uB[1] = lb.U[1] + (W2 * rb[0] - W0 * rb[2]);
+    uB[2] = lb.U[2] + (W0 * rb[1] - W1 * rb[0]);
+    const float drF = mF.x;
+    const float uF[3] = {mF.y, mF.z, mF.w};
+    // stability check at the fluid end of every cut link: a NaN or
+    // |u| > 0.3 marks the solve unstable (counters[5]; LBM_ERR_UNSTABLE)
+    if (!(uF[0] * uF[0] + uF[1] * uF[1] + uF[2] * uF[2] < 0.09f)) atomicOr(&sb.counters[5], 1ull);
+    float ubf[3], chi;
+    if (dl < 0.5f) {
+        if (G >= 0) {
+            ubf[0] = mG.y;
+            ubf[1] = mG.z;
+            ubf[2] = mG.w;
+            chi = (2.0f * dl - 1.0f) / (p.tauf - 2.0f);
         } else {
-            double k3 = 3.0 / (2.0 * delta);
-            for (int a = 0; a < 3; ++a) ubf[a] = uF[a] + k3 * (uB[a] - uF[a]);
-            chi = (2.0 * delta - 1.0) / (p.tau + 0.5);
+            ubf[0] = uF[0];
+            ubf[1] = uF[1];
+            ubf[2] = uF[2];
+            chi = 0.0f;
         }
-        double g = geq_x(p, tb, ib, rhoF, ubf, uF);
-        double rhow = p.eq == 0 ? p.rho0 : rhoF;
-        double cuB = (double)cxi * uB[0] + (double)cyi * uB[1] + (double)czi * uB[2];
-        double bc = (1.0 - chi) * fb + chi * g + 2.0 * tb.w[i] * rhow * 3.0 * cuB;
-        stS(pop + (long long)i * N + A, bc);
-        fa = bc;
-        double sum = fa + fb;
-        ps[0] = -cxi * sum;
-        ps[1] = -cyi * sum;
-        ps[2] = -czi * sum;
-        const int cb[3] = {-cxi, -cyi, -czi};
-        const int cc[3] = {cxi, cyi, czi};
-        for (int a = 0; a < 3; ++a) pm[a] = -(cc[a] - uB[a]) * fa + (cb[a] - uB[a]) * fb;
     } else {
-        const float fbf = ldP(pop + (long long)ib * N + cell);
-        // moments of f(t) at x_F (and at x_F + c_i): kept by the previous
-        // stream-collide pass (or the refill, or the initial state)
-        const float *macf = (const float *)sb.mac_t;
-        const float4 mF = load_mac(macf, cell);
-        const float drF = mF.x;
-        const float uF[3] = {mF.y, mF.z, mF.w};
-        // stability check at the fluid end of every cut link: a NaN or
-        // |u| > 0.3 marks the solve unstable (counters[5]; LBM_ERR_UNSTABLE)
-        if (!(uF[0] * uF[0] + uF[1] * uF[1] + uF[2] * uF[2] < 0.09f)) atomicOr(&sb.counters[5], 1ull);
-        float ubf[3], chi;
-        const float dl = (float)delta;
-        if (delta < 0.5) {
-            if (G >= 0) {
-                ubf[0] = mG.y;
-                ubf[1] = mG.z;
-                ubf[2] = mG.w;
-                chi = (2.0f * dl - 1.0f) / ((float)p.tau - 2.0f);
-            } else {
-                ubf[0] = uF[0];
-                ubf[1] = uF[1];
-                ubf[2] = uF[2];
-                chi = 0.0f;
-            }
-        } else {
-            const float k3 = 3.0f / (2.0f * dl);
-            for (int a = 0; a < 3; ++a) ubf[a] = fmaf(k3, (float)uB[a] - uF[a], uF[a]);
-            chi = (2.0f * dl - 1.0f) / ((float)p.tau + 0.5f);
-        }
-        const float g = dgeq_f(p, tb, ib, drF, ubf, uF);
-        const float rhow = p.eq == 0 ? p.rho0f : 1.0f + drF;
-        const float cuB = cxi * (float)uB[0] + cyi * (float)uB[1] + czi * (float)uB[2];
-        const float bc = fmaf(6.0f * (float)tb.w[i] * rhow, cuB, fmaf(chi, g - fbf, fbf));
-        stS(pop + (long long)i * N + A, bc);
-        fa = (double)roundS(pop, bc);
-        fb = (double)fbf;
-        // deviation form: the constant parts -2 w_i c_i cancel over the
-        // closed link set of a body (N_i = N_ib on every lattice line);
-        // per-link products in FP32, the per-body sums in FP64
-        const float sum = (float)fa + fbf, dif = (float)fa - fbf;
-        const float d0 = (float)d[0], d1 = (float)d[1], d2 = (float)d[2];
-        const float s0 = -cxi * sum, s1 = -cyi * sum, s2 = -czi * sum;
-        const float m0 = fmaf((float)uB[0], dif, s0), m1 = fmaf((float)uB[1], dif, s1),
-                    m2 = fmaf((float)uB[2], dif, s2);
-        outf[0] = s0;
-        outf[1] = s1;
-        outf[2] = s2;
-        outf[3] = d1 * s2 - d2 * s1;
-        outf[4] = d2 * s0 - d0 * s2;
-        outf[5] = d0 * s1 - d1 * s0;
-        outf[6] = m0;
-        outf[7] = m1;
-        outf[8] = m2;
-        outf[9] = d1 * m2 - d2 * m1;
-        outf[10] = d2 * m0 - d0 * m2;
-        outf[11] = d0 * m1 - d1 * m0;
-        return;
+        const float k3 = 3.0f / (2.0f * dl);
+        for (int a = 0; a < 3; ++a) ubf[a] = fmaf(k3, uB[a] - uF[a], uF[a]);
+        chi = (2.0f * dl - 1.0f) / (p.tauf + 0.5f);
     }
-    double ts[3], tm[3];
-    cross3(d, ps, ts);
-    cross3(d, pm, tm);
-    out[0] = ps[0];
-    out[1] = ps[1];
-    out[2] = ps[2];
-    out[3] = ts[0];
-    out[4] = ts[1];
-    out[5] = ts[2];
-    out[6] = pm[0];
-    out[7] = pm[1];
-    out[8] = pm[2];
-    out[9] = tm[0];
-    out[10] = tm[1];
-    out[11] = tm[2];
+    const float g = dgeq_f(p, tb, wf, ib, drF, ubf, uF);
+    const float rhow = p.eq == 0 ? p.rho0f : 1.0f + drF;
+    const float cuB = cxi * uB[0] + cyi * uB[1] + czi * uB[2];
+    const float bc = fmaf(6.0f * wf[i] * rhow, cuB, fmaf(chi, g - fb, fb));
+    stS(pop + (long long)i * N + A, bc);
+    const float fa = roundS(pop, bc);
+    // deviation form: the constant parts -2 w_i c_i cancel over the
+    // closed link set of a body (N_i = N_ib on every lattice line);
+    // per-link products in FP32, the per-body sums exact
+    const float sum = fa + fb, dif = fa - fb;
+    const float s0 = -cxi * sum, s1 = -cyi * sum, s2 = -czi * sum;
+    const float m0 = fmaf(uB[0], dif, s0), m1 = fmaf(uB[1], dif, s1), m2 = fmaf(uB[2], dif, s2);
+    out[0] = s0;
+    out[1] = s1;
+    out[2] = s2;
+    out[3] = d[1] * s2 - d[2] * s1;
+    out[4] = d[2] * s0 - d[0] * s2;
+    out[5] = d[0] * s1 - d[1] * s0;
+    out[6] = m0;
+    out[7] = m1;
+    out[8] = m2;
+    out[9] = d[1] * m2 - d[2] * m1;
+    out[10] = d[2] * m0 - d[0] * m2;
+    out[11] = d[0] * m1 - d[1] * m0;
 }
 
 // this thread's entry of the run-time table (the whole block calls it)
@@ -1274,8 +1295,7 @@ __global__ void __launch_bounds__(LINK_THREADS) k_links(Params p, StepBufs sb) {
             const double *X = sb.poses + (long long)b * POSE_STRIDE + 3;
             const long long j = B.link_off + (k - sb.link_pre[b]);
             double out[ME_PER_LINK];
-            float outf[ME_PER_LINK];
-            link_work<L, P>(p, sb, tb, B, X, j, out, outf);
+            link_exact<L, P>(p, sb, tb, B, X, j, out);
             const long long st = p.me_stride;
             for (int c = 0; c < ME_PER_LINK; ++c) sb.me[c * st + j] = out[c];
         }
@@ -1283,6 +1303,9 @@ __global__ void __launch_bounds__(LINK_THREADS) k_links(Params p, StepBufs sb) {
         // tile -> body map in shared memory (binary search), global beyond 1024 bodies
         __shared__ long long tp_s[1025];
         __shared__ unsigned long long part[LINK_THREADS / 32][ME_PER_LINK];
+        __shared__ LinkBody lb;
+        __shared__ float wf[L::Q];
+        if (threadIdx.x < L::Q) wf[threadIdx.x] = L::template w<float>(threadIdx.x);
         const bool in_smem = p.nb < 1025;
         if (in_smem)
             for (int k = threadIdx.x; k <= p.nb; k += blockDim.x) tp_s[k] = sb.tile_pre[k];
@@ -1302,10 +1325,11 @@ __global__ void __launch_bounds__(LINK_THREADS) k_links(Params p, StepBufs sb) {
             const long long k = (tile - tp[b]) * LINK_THREADS + threadIdx.x;
             // appended lists count past a full segment; only its links exist
             const long long cnt = min(sb.link_cnt[b], B.link_cap);
-            double out[ME_PER_LINK];
+            fill_link_body(lb, B, X);
+            __syncthreads();
             float outf[ME_PER_LINK];
             for (int c = 0; c < ME_PER_LINK; ++c) outf[c] = 0.0f;
-            if (k < cnt) link_work<L, P>(p, sb, tb, B, X, B.link_off + k, out, outf);
+            if (k < cnt) link_fast<L, P>(p, sb, tb, wf, lb, B.link_off + k, outf);
             // the tile's sums: warp shuffles, then one atomic per block and
             // component (every tile of a body adds into the same 12 words)
             const int wid = threadIdx.x >> 5;
