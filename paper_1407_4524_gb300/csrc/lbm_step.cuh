@@ -1584,27 +1584,42 @@ __device__ __forceinline__ void imp_body_fast(const Params &p, const StepBufs &s
             double r1[3], uBd[3];
             disp(p, X1, x, y, z, r1);
             body_velocity(B, r1, uBd);
+            // the neighbours in batches whose loads are in flight together (a
+            // load a neighbour behind the test of its owner waits 36 times: the
+            // 151x97x84 moving spheres' step 66.7 -> 59.2 us)
             float sum = 0.f, us[3] = {0.f, 0.f, 0.f};
             int nn = 0;
+            constexpr int BATCH = 6;
 #pragma unroll
-            for (int i = 1; i < L::Q; ++i) {
-                int q[3] = {x + L::cx(i), y + L::cy(i), z + L::cz(i)};
-                const int n[3] = {p.nx, p.ny, p.nz};
-                bool ok = true;
-                for (int a = 0; a < 3; ++a) {
-                    if (q[a] >= 0 && q[a] < n[a]) continue;
-                    if (!p.per[a]) ok = false;
-                    else q[a] += q[a] < 0 ? n[a] : -n[a];
+            for (int i0 = 1; i0 < L::Q; i0 += BATCH) {
+                bool use[BATCH];
+                float4 m[BATCH]; // moments of f(t)
+#pragma unroll
+                for (int k = 0; k < BATCH; ++k) {
+                    const int i = i0 + k;
+                    if (i >= L::Q) continue;
+                    int q[3] = {x + L::cx(i), y + L::cy(i), z + L::cz(i)};
+                    const int n[3] = {p.nx, p.ny, p.nz};
+                    bool ok = true;
+                    for (int a = 0; a < 3; ++a) {
+                        if (q[a] >= 0 && q[a] < n[a]) continue;
+                        if (!p.per[a]) ok = false;
+                        else q[a] += q[a] < 0 ? n[a] : -n[a];
+                    }
+                    const long long nb = ok ? cell_of(p, q[0], q[1], q[2]) : A;
+                    const uint16_t o = sb.owner_t[nb];
+                    m[k] = load_mac((const float *)sb.mac_t, nb);
+                    use[k] = ok && o == 0;
                 }
-                if (!ok) continue;
-                const long long nb = cell_of(p, q[0], q[1], q[2]);
-                if (sb.owner_t[nb] != 0) continue;
-                const float4 m = load_mac((const float *)sb.mac_t, nb); // moments of f(t)
-                sum += m.x;
-                us[0] += m.y;
-                us[1] += m.z;
-                us[2] += m.w;
-                nn++;
+#pragma unroll
+                for (int k = 0; k < BATCH; ++k) {
+                    if (i0 + k >= L::Q || !use[k]) continue;
+                    sum += m[k].x;
+                    us[0] += m[k].y;
+                    us[1] += m[k].z;
+                    us[2] += m[k].w;
+                    nn++;
+                }
             }
             long long ec[3];
             if (p.refill == 2 && extrap_cells<L>(p, B, X1, sb.owner_t, x, y, z, ec) != 0) {
