@@ -2015,6 +2015,7 @@ int batch_rebuild(lbm_batch *B) {
                 sbuf.mac_t = D->mac[par];
                 sbuf.mac_t1 = D->mac[par ^ 1];
                 sbuf.flags = D->flags;
+                sbuf.counters = D->counters; // (the kernel on bulk-copied tiles reports expired waits there)
                 const int b = q % nbr;
                 e = launch_bulk(D->Q, D->prec, D->p, sbuf, b == 0 ? B->s : B->sb[b - 1]);
             }
