@@ -768,7 +768,10 @@ int do_step(lbm_domain *D) {
     };
     StepBufs sb = step_bufs(D);
     GeomArgs g = geom_args(D, true);
-    g.grid_cap = side ? 2 * D->side_blocks : 0; // (blocks of half the threads of the other kernels' cap)
+    // four times the other side kernels' cap: the longer the geometry takes, the
+    // longer it holds room the pass could use (512x256x256 swarm's step with 1, 2,
+    // 4 blocks an SM: FP32 819, 802, 798 us, FP16 468, 450, 440 us)
+    g.grid_cap = side ? 4 * D->side_blocks : 0;
     CK(wait(s2, D->ev_prep, D->s));
     if (D->n_moving) {
         if ((rc = geometry_owners(D, g, s2))) return rc;
