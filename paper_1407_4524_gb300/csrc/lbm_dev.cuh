@@ -19,9 +19,9 @@
 namespace lbm {
 
 constexpr uint8_t FL_SOLID = 1; // node inside a body at time t
-constexpr uint8_t FL_MAC = 2;   // store rho,u of f(t+1) at this node (FP64 mode)
+constexpr uint8_t FL_MAC = 2;   // store rho,u of f(t+1) at this node
 constexpr uint8_t FL_BND = 4;   // fluid node with a solid neighbour at t (handled by
-                                // the boundary-node kernel in the reduced-precision modes)
+                                // the boundary-node kernel in served solves)
 
 constexpr int SERIES_ROW = 18;  // Fs Ts Fi Ti Fm Tm
 constexpr int ME_PER_LINK = 12; // Fs Ts Fm Tm contributions of one link
@@ -149,6 +149,7 @@ struct Params {
     int pair;    // reduced precision: two nodes per thread where that kernel applies
     int stage_expire_test; // test hook: the staged kernel issues no copy, so its waits expire
     int nsm;     // multiprocessors of the device
+    int z0, zc;  // stream-collide of the zc planes from z0 on (wrapping) only; zc = 0: all
     int zouhe;   // wall / inlet faces are Zou-He nodes (else half-way links)
     int free_scheme; // covered / uncovered sets of free bodies: 0 explicit, 1 backward sets
                      // of the previous displacement, 2 predictor-corrector

@@ -33,7 +33,7 @@ inline dim3 bulk_block(const Params &p) {
 
 inline dim3 bulk_grid(const Params &p) {
     dim3 b = bulk_block(p);
-    return dim3((p.nx + b.x - 1) / b.x, p.ny, p.nz);
+    return dim3((p.nx + b.x - 1) / b.x, p.ny, p.zc ? p.zc : p.nz);
 }
 
 template <class L, class P>

@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, pair_min_blocks<P>()) k_bulk_pai
                                                             typename P::S *__restrict__ dst,
                                                             const uint8_t *__restrict__ flags,
                                                             typename P::C *__restrict__ mac_t1) {
-    pair_nodes<L, P>(p, src, dst, flags, mac_t1, 2 * (blockIdx.x * blockDim.x + threadIdx.x), blockIdx.y, blockIdx.z);
+    pair_nodes<L, P>(p, src, dst, flags, mac_t1, 2 * (blockIdx.x * blockDim.x + threadIdx.x), blockIdx.y, bulk_plane(p));
 }
 
 // the pair kernel's conditions: no body force, nx even, every axis periodic,
@@ -277,7 +277,7 @@ inline dim3 pair_block(const Params &p) {
 
 inline dim3 pair_grid(const Params &p) {
     const dim3 b = pair_block(p);
-    return dim3((p.nx / 2 + b.x - 1) / b.x, p.ny, p.nz);
+    return dim3((p.nx / 2 + b.x - 1) / b.x, p.ny, p.zc ? p.zc : p.nz);
 }
 
 } // namespace lbm

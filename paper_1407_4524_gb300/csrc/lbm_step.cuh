@@ -5,7 +5,7 @@
 // Storage convention: the population buffer of step t holds the
 // post-collision values fhat(x, t) (Eq. collision) at every fluid node.
 //
-// FP64 mode (parity), one stream, per step:
+// Per step (streams: do_step in lbm_api.cu):
 //   k_links  : for every cut link (x_F fluid, x_A = x_F - c_i solid) the wall
 //              value fhat_i(x_A, t) of Eq. Fillipova_interpolation, stored in
 //              the (otherwise unused) slot i of the solid node x_A, and the
@@ -13,20 +13,19 @@
 //              flow_torque_2, ForceInMovementMovingFrame,
 //              TorqueInMovementMovingFrame), which by Eq. Equalities need
 //              exactly that wall value and fhat_ib(x_F, t);
-//   k_bulk   : pull-streaming f_i(x, t+1) = fhat_i(x - c_i, t) (Eq.
-//              streaming) -- at cut links the pull reads the wall value --,
-//              moments (Eqs. LBMmacroscopics_0/1), BGK collision, store;
-//   k_finish : per-body sums of the link contributions in link order into the
-//              force/torque row of step t; for moving bodies the covered /
-//              uncovered nodes A+ / A- (Sec. 3.2.2): impulsive terms of Eqs.
-//              ForceInMovement / TorqueInMovement, refill of uncovered nodes.
-// Every formula there has the FP64 CPU oracle's operation order, so the FP64
-// mode reproduces it bit for bit.
-//
-// FP32 / FP16 modes: k_bulk skips the boundary nodes (fluid nodes with a solid
-// neighbour), which the boundary-node kernel (lbm_bnd.cuh) steps on a second
-// stream; k_finish converts the exact fixed-point per-body sums.  Storage is
-// f - w, arithmetic FP32.
+//   k_bulk   : (or k_bulk_pair, k_bulk_tma) pull-streaming f_i(x, t+1) =
+//              fhat_i(x - c_i, t) (Eq. streaming) -- at cut links the pull
+//              reads the wall value --, moments (Eqs. LBMmacroscopics_0/1),
+//              BGK collision, store;
+//   k_finish : the force/torque row of step t of every body; for moving
+//              bodies the covered / uncovered nodes A+ / A- (Sec. 3.2.2):
+//              impulsive terms of Eqs. ForceInMovement / TorqueInMovement,
+//              refill of uncovered nodes.
+// FP64 mode (parity): every formula has the FP64 CPU oracle's operation order
+// (per-body sums in link order), so it reproduces the oracle bit for bit.
+// FP32 / FP16 modes: storage is f - w, arithmetic FP32, the per-body sums exact
+// fixed point.  A served solve's pass skips the boundary nodes (fluid nodes
+// with a solid neighbour), which the boundary-node kernel (lbm_bnd.cuh) steps.
 //
 // Every mode: under the Zou-He edge rule k_bulk also skips the nodes of the
 // wall and inlet faces, which k_zouhe steps (pull, closure of the entering
@@ -969,6 +968,12 @@ __device__ __forceinline__ void bulk_node(const Params &p, const typename P::S *
     for (int i = 0; i < L::Q; ++i) stS(dst + (size_t)N32 * (unsigned)i + c32, f[i]);
 }
 
+// the plane of a block of the stream-collide kernels
+__device__ __forceinline__ int bulk_plane(const Params &p) {
+    const int z = (int)blockIdx.z + p.z0;
+    return z >= p.nz ? z - p.nz : z;
+}
+
 // pull-stream + moments + BGK collision over every fluid node
 template <class L, class P, int FM>
 __global__ void __launch_bounds__(BULK_THREADS, P::exact ? 4 : bulk_min_blocks<FM>()) k_bulk(Params p, const typename P::S *__restrict__ src,
@@ -976,7 +981,7 @@ __global__ void __launch_bounds__(BULK_THREADS, P::exact ? 4 : bulk_min_blocks<F
                                                        const uint8_t *__restrict__ flags,
                                                        const typename P::C *__restrict__ mac_t,
                                                        typename P::C *__restrict__ mac_t1) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, z = bulk_plane(p);
     if (x >= p.nx) return;
     bulk_node<L, P, FM>(p, src, dst, flags, mac_t, mac_t1, x, y, z);
 }
