@@ -18,6 +18,7 @@
 // even.
 #pragma once
 
+#include "lbm_cols.h"
 #include "lbm_step.cuh"
 
 namespace lbm {
@@ -188,7 +189,8 @@ __device__ __forceinline__ void pair_nodes(const Params &p, const typename P::S 
     const int lane = threadIdx.x & 31;
     const int nx = p.nx;
     const bool valid = x0 < nx;
-    const int xc = valid ? x0 : nx - 2; // lanes past the row load in bounds, store nothing
+    const PairCols col = pair_cols(x0, nx); // lanes past the row load in bounds, store nothing
+    const int xc = col.own;
     const unsigned ny = (unsigned)p.ny, N32 = (unsigned)p.N;
     const unsigned cell0 = ((unsigned)z * ny + (unsigned)y) * (unsigned)nx + (unsigned)xc;
     const unsigned fl2 = __ldg(reinterpret_cast<const unsigned short *>(flags + cell0));
@@ -201,8 +203,7 @@ __device__ __forceinline__ void pair_nodes(const Params &p, const typename P::S 
     const int zm = z == 0 ? p.nz - 1 : z - 1, zp = z == p.nz - 1 ? 0 : z + 1;
     // the element left of x0 (lane 0) and the pair right of x0 + 1 (lane 31,
     // or the row's last pair): periodic along x where these are used
-    const int xl = (x0 == 0 ? nx : x0) - 2; // pair holding x0 - 1 as element 1
-    const int xr = x0 + 2 >= nx ? 0 : x0 + 2;
+    const int xl = col.left, xr = col.right;
     const bool ld_l = lane == 0, ld_r = lane == 31 || x0 + 2 >= nx;
     F2 f[L::Q];
 #pragma unroll
