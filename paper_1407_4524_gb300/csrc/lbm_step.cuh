@@ -912,8 +912,16 @@ __global__ void __launch_bounds__(BULK_THREADS) k_macros(Params p, const typenam
                 if (c[a] == -1) j[a] -= v;
             }
         }
-        if (!finite_x(r)) // a population is not finite: so is every component (0 * inf)
-            for (int a = 0; a < 3; ++a) j[a] += 0.0 * r;
+        if (!finite_x(r)) { // a population, or a sum of them, is not finite: every product counts (0 * inf is NaN)
+            for (int a = 0; a < 3; ++a) j[a] = 0.0;
+            for (int i = 0; i < L::Q; ++i) {
+                double v = (double)ldS(src + (long long)i * p.N + cell);
+                if constexpr (!P::exact) v += L::template w<double>(i);
+                j[0] += (double)L::cx(i) * v;
+                j[1] += (double)L::cy(i) * v;
+                j[2] += (double)L::cz(i) * v;
+            }
+        }
         for (int a = 0; a < 3; ++a) j[a] = j[a] - 0.5 * p.g[a];
         if (p.eq != 0 || p.rho0 != 1.0) {
             const double den = p.eq == 0 ? p.rho0 : r;
