@@ -487,6 +487,15 @@ __device__ __noinline__ typename P::C pull_edge(const Params &p, const typename 
     return ldS(src + (long long)i * p.N + cell_of(p, s[0], s[1], s[2]));
 }
 
+// 1 + the sum of the deviations fhat - w of a node (reduced precision)
+template <class L, class S>
+__device__ __forceinline__ float own_density(const Params &p, const S *__restrict__ src, long long cell) {
+    float r = 0.0f;
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) r += ldP(src + (long long)i * p.N + cell);
+    return 1.0f + r;
+}
+
 // Momentum terms of the wall / inlet links of one node (Delta = 1/2, chi = 0:
 // moving bounce-back, u_B = 0 on walls, the inlet profile on inlet links; a
 // wall wins at corners) -- the same expressions as pull_edge.
@@ -505,7 +514,12 @@ __device__ __forceinline__ void face_terms(const Params &p, const typename P::S 
             f[i] = f[i] + 2.0 * L::template w<double>(i) * rhow * 3.0 * cuB;
         }
     } else {
-        if (!inlet_only) return; // walls at rest: the bounced population as it is
+        if (!inlet_only) { // walls at rest: the bounced population as it is
+            // (standard model: the term is 0 times the node's own density, which
+            // leaves no population of the node finite where it is not itself)
+            if (p.eq != 0) f[0] += 0.0f * own_density<L>(p, src, cell);
+            return;
+        }
         float rhow = p.rho0f;
         if (p.eq != 0) {
             float dr, uu[3];
