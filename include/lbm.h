@@ -52,8 +52,14 @@ extern "C" {
 #define LBM_ERR_CUDA 3     /* a CUDA runtime call failed (message has the reason) */
 #define LBM_ERR_UNSTABLE 4 /* a NaN or |u| > 0.3 was detected in a checked step
                              (returned by the series / force reads of that solve) */
-#define LBM_ERR_TIMEOUT 5  /* a bounded device wait gave up (the mbarrier waits of
-                             the staged stream-collide kernel, LBM_STAGED=1) */
+#define LBM_ERR_TIMEOUT 5  /* a bounded device wait gave up in some step so far (the
+                             mbarrier waits of the stream-collide kernels that bring
+                             their rows by bulk copies: large LBM_FP16 domains, and
+                             LBM_STAGED=1), so nodes were left unstepped: every read
+                             of results returns it (series, force / torque,
+                             populations, moments, body state, solid owners,
+                             snapshots; lbm_get_stats counts it instead).  Loading
+                             a snapshot taken before it clears it */
 #define LBM_ERR_STATE 6    /* call not allowed in the current state */
 
 /* ---- enumerations -------------------------------------------------------------- */

@@ -1412,6 +1412,20 @@ int wait_steps(lbm_domain *D, int64_t t_end) {
     }
     return LBM_OK;
 }
+
+int fail_expired() {
+    return fail(LBM_ERR_TIMEOUT, "a stream-collide block gave up waiting for its rows: nodes were left unstepped");
+}
+
+// Every read of state that the steps so far made: LBM_ERR_TIMEOUT when a
+// bounded wait ran out in one of them (the sticky flag of the stream-collide
+// kernels that bring their rows by bulk copies).  Waits for the domain's stream.
+int check_waits(lbm_domain *D) {
+    unsigned long long expired = 0;
+    CK(cudaMemcpyAsync(&expired, D->counters + 6, sizeof(expired), cudaMemcpyDeviceToHost, D->s));
+    CK(cudaStreamSynchronize(D->s));
+    return expired ? fail_expired() : LBM_OK;
+}
 } // namespace
 
 int lbm_get_series(lbm_domain *D, int64_t first, int64_t count, double *out) {
@@ -1419,7 +1433,7 @@ int lbm_get_series(lbm_domain *D, int64_t first, int64_t count, double *out) {
     DEVICE_SCOPE(D->d.device);
     if (first + count > D->t) return fail(LBM_ERR_ARG, "rows beyond the current step");
     if (first < D->t - D->series_cap) return fail(LBM_ERR_ARG, "rows older than the series ring");
-    if (D->nb == 0 || count == 0) return LBM_OK;
+    if (count == 0) return LBM_OK;
     int wrc = wait_steps(D, first + count);
     if (wrc) return wrc;
     {
@@ -1428,7 +1442,7 @@ int lbm_get_series(lbm_domain *D, int64_t first, int64_t count, double *out) {
         unsigned long long flags[3] = {0, 0, 0}; // unstable, timeout, free body out of range
         CK(cudaMemcpyAsync(flags, D->counters + 5, sizeof(flags), cudaMemcpyDeviceToHost, D->sio));
         CK(cudaStreamSynchronize(D->sio));
-        if (flags[1]) return fail(LBM_ERR_TIMEOUT, "a stream-collide block gave up waiting for its staged rows");
+        if (flags[1]) return fail_expired();
         if (flags[0])
             return fail(LBM_ERR_UNSTABLE, "the solve went unstable (NaN or |u| > 0.3 at a boundary node, or a "
                                           "non-finite force)");
@@ -1436,6 +1450,7 @@ int lbm_get_series(lbm_domain *D, int64_t first, int64_t count, double *out) {
             return fail(LBM_ERR_STATE, "a free body came within 2 cells of a non-periodic face or moved faster "
                                        "than 0.25 at its surface");
     }
+    if (D->nb == 0) return LBM_OK; // no rows
     const size_t row = (size_t)D->nb * SERIES_ROW;
     int64_t done = 0;
     while (done < count) {
@@ -1523,7 +1538,7 @@ int lbm_get_populations(lbm_domain *D, double *out) {
     if (e == cudaSuccess) e = cudaMemcpy(out, tmp, n * sizeof(double), cudaMemcpyDeviceToHost);
     D->release(tmp);
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, std::string("populations: ") + cudaGetErrorString(e));
-    return LBM_OK;
+    return check_waits(D);
 }
 
 // cells of the staging buffer of lbm_set_populations / lbm_get_macros
@@ -1588,7 +1603,7 @@ int lbm_get_macros(lbm_domain *D, double *out) {
     D->release(stage);
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, std::string("macros: ") + cudaGetErrorString(e));
     D->d2h += N * 4 * (long long)sizeof(double);
-    return LBM_OK;
+    return check_waits(D);
 }
 
 int lbm_get_body_state(lbm_domain *D, double *out) {
@@ -1596,7 +1611,7 @@ int lbm_get_body_state(lbm_domain *D, double *out) {
     DEVICE_SCOPE(D->d.device);
     if (D->nb == 0) return LBM_OK;
     std::vector<BodyDev> hb((size_t)D->nb);
-    CK(cudaStreamSynchronize(D->s));
+    if (int rc = check_waits(D)) return rc;
     CK(cudaMemcpy(hb.data(), D->dbodies, sizeof(BodyDev) * D->nb, cudaMemcpyDeviceToHost));
     D->d2h += (long long)(sizeof(BodyDev) * D->nb);
     for (int b = 0; b < D->nb; ++b) {
@@ -1611,15 +1626,22 @@ int lbm_get_body_state(lbm_domain *D, double *out) {
     return LBM_OK;
 }
 
-int lbm_get_solid(lbm_domain *D, int32_t *out) {
-    if (!D || !out) return fail(LBM_ERR_ARG, "invalid arguments");
-    DEVICE_SCOPE(D->d.device);
+namespace {
+int read_solid(lbm_domain *D, int32_t *out) {
     const size_t N = (size_t)D->p.N;
     std::vector<uint16_t> o(N);
     CK(cudaStreamSynchronize(D->s));
     CK(cudaMemcpy(o.data(), D->owner[D->t & 1], N * sizeof(uint16_t), cudaMemcpyDeviceToHost));
     for (size_t k = 0; k < N; ++k) out[k] = (int32_t)o[k] - 1;
     return LBM_OK;
+}
+} // namespace
+
+int lbm_get_solid(lbm_domain *D, int32_t *out) {
+    if (!D || !out) return fail(LBM_ERR_ARG, "invalid arguments");
+    DEVICE_SCOPE(D->d.device);
+    if (int rc = check_waits(D)) return rc;
+    return read_solid(D, out);
 }
 
 // ---- state snapshots --------------------------------------------------------
@@ -1650,7 +1672,7 @@ int lbm_save_state(lbm_domain *D, void *out, int64_t cap) {
     DEVICE_SCOPE(D->d.device);
     const int64_t need = lbm_state_bytes(D);
     if (cap < need) return fail(LBM_ERR_ARG, "snapshot buffer smaller than lbm_state_bytes");
-    CK(cudaStreamSynchronize(D->s));
+    if (int rc = check_waits(D)) return rc;
     char *p = (char *)out;
     SnapHeader h{};
     std::memcpy(h.magic, SNAP_MAGIC, 8);
@@ -1759,7 +1781,7 @@ int lbm_get_stats(lbm_domain *D, lbm_stats *out) {
         for (long long v : lc) out->links += v;
     }
     std::vector<int32_t> s((size_t)D->p.N);
-    int rc = lbm_get_solid(D, s.data());
+    int rc = read_solid(D, s.data());
     if (rc) return rc;
     for (int32_t v : s) out->fluid_cells += v < 0;
     return LBM_OK;
@@ -2408,6 +2430,5 @@ extern "C" int lbm_get_populations_noalloc(lbm_domain *D, double *out) {
     DEVICE_SCOPE(dev);
     CK(launch_export(D->Q, D->prec, D->p, D->pop[D->t & 1], scratch, D->s));
     CK(cudaMemcpyAsync(out, scratch, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, D->s));
-    CK(cudaStreamSynchronize(D->s));
-    return LBM_OK;
+    return check_waits(D);
 }
