@@ -25,14 +25,14 @@
 #pragma once
 
 #include "lbm_step.cuh"
+#include "lbm_wait.h"
 
 namespace lbm {
 
 constexpr int STAGE_SEG = 256;        // nodes per segment (threads per block) at most
 constexpr int STAGE_BLOCKS_PER_SM = 4;
 constexpr unsigned long long LBM_TIMEOUT_FLAG = 1ull;
-constexpr unsigned long long STAGE_WAIT_NS = 1000000000ull; // a wait gives up after one second
-constexpr long long STAGE_WAIT_ROUNDS = 1ll << 24;             // and after this many poll rounds at most
+constexpr long long STAGE_WAIT_ROUNDS = 1ll << 24; // a wait gives up after this many poll rounds at most
 
 __device__ __forceinline__ unsigned smem_u32(const void *ptr) {
     return (unsigned)__cvta_generic_to_shared(ptr);
@@ -66,15 +66,15 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-// bounded wait for the phase of the given parity (one second, and a round
-// count); false if it never completed
+// bounded wait for the phase of the given parity (one second of polling, and a
+// round count); false if it never completed
 __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *bar, unsigned parity) {
     if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
+    WaitClock c{global_ns(), 0ull};
     for (long long r = 0; r < STAGE_WAIT_ROUNDS; ++r) {
         for (int k = 0; k < 64; ++k)
             if (mbar_try_wait(bar, parity)) return true;
-        if (global_ns() - t0 > STAGE_WAIT_NS) return false;
+        if (wait_over(c, global_ns())) return false;
     }
     return false;
 }
