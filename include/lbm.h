@@ -370,8 +370,8 @@ int lbm_get_macros(lbm_domain *dom, double *out);
  * same descriptor and given the same number of bodies by lbm_set_bodies, so
  * that its buffers have the snapshot's sizes (LBM_ERR_ARG otherwise); the
  * steps that follow reproduce those of the saved domain bit for bit.
- * A snapshot is raw host-endian memory of this library version: it is not a
- * portable file format.  Every check runs before anything is changed, so
+ * A snapshot is raw host-endian memory: it is not a portable file format.  One
+ * that an earlier version of the library wrote is accepted.  Every check runs before anything is changed, so
  * LBM_ERR_ARG leaves the domain as it was; after LBM_ERR_CUDA its state is
  * undefined (load the snapshot again or destroy the domain).  Synchronises. */
 int64_t lbm_state_bytes(const lbm_domain *dom);

@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -130,6 +131,18 @@ struct DevGuard {
 
 } // namespace
 
+// A persistent device buffer, as a state snapshot holds it
+enum StateKind {
+    STATE_DATA,    // its contents, of the same size in every version of the library
+    STATE_BODIES,  // the bodies' records, which have grown
+    STATE_DERIVED, // made anew from the bodies' records: contents and size are the writer's own
+};
+struct StateBuf {
+    void *ptr;
+    size_t n;
+    StateKind kind;
+};
+
 struct lbm_domain {
     lbm_domain_desc d{};
     Params p{};
@@ -151,11 +164,12 @@ struct lbm_domain {
     std::vector<void *> body_allocs;
     // every persistent device buffer with its size, in allocation order: the
     // device part of a state snapshot (lbm_save_state / lbm_load_state)
-    std::vector<std::pair<void *, size_t>> state_bufs;
+    std::vector<StateBuf> state_bufs;
     BodyDev *dbodies = nullptr;
     int *dmoving = nullptr;
     int2 *chunk_all = nullptr, *chunk_mov = nullptr;
     int nchunk_all = 0, nchunk_mov = 0;
+    size_t chunk_cap = 0; // entries of each
     int *chunk_cnt_apm = nullptr, *chunk_cnt_link = nullptr;
     uint32_t *Lcell[2] = {nullptr, nullptr};
     uint8_t *Ldir[2] = {nullptr, nullptr};
@@ -251,20 +265,21 @@ struct lbm_domain {
 
 namespace {
 
-int alloc_into(lbm_domain *D, void **slot, size_t n, std::vector<void *> *track) {
+int alloc_into(lbm_domain *D, void **slot, size_t n, std::vector<void *> *track, StateKind kind = STATE_DATA) {
     void *ptr = D->alloc(n);
     if (!ptr) return fail(LBM_ERR_OOM, "device allocation of " + std::to_string(n) + " bytes failed");
     D->bytes += n;
     if (cudaMemsetAsync(ptr, 0, n, D->s) != cudaSuccess) return fail(LBM_ERR_CUDA, "cudaMemsetAsync failed");
     *slot = ptr;
     if (track) track->push_back(ptr);
-    D->state_bufs.emplace_back(ptr, n);
+    D->state_bufs.push_back({ptr, n, kind});
     return LBM_OK;
 }
 
-template <class T> int alloc_t(lbm_domain *D, T **slot, size_t count, std::vector<void *> *track) {
+template <class T>
+int alloc_t(lbm_domain *D, T **slot, size_t count, std::vector<void *> *track, StateKind kind = STATE_DATA) {
     void *v = nullptr;
-    int rc = alloc_into(D, &v, count * sizeof(T), track);
+    int rc = alloc_into(D, &v, count * sizeof(T), track, kind);
     *slot = (T *)v;
     return rc;
 }
@@ -272,7 +287,7 @@ template <class T> int alloc_t(lbm_domain *D, T **slot, size_t count, std::vecto
 void free_body_buffers(lbm_domain *D) {
     for (void *ptr : D->body_allocs) {
         for (size_t k = 0; k < D->state_bufs.size(); ++k)
-            if (D->state_bufs[k].first == ptr) {
+            if (D->state_bufs[k].ptr == ptr) {
                 D->state_bufs.erase(D->state_bufs.begin() + (long)k);
                 break;
             }
@@ -321,6 +336,7 @@ void free_body_buffers(lbm_domain *D) {
     D->nb = D->n_moving = D->n_free = 0;
     D->split_n = 0;
     D->nchunk_all = D->nchunk_mov = 0;
+    D->chunk_cap = 0;
     D->link_cap_total = D->apm_cap_total = 0;
 }
 
@@ -349,6 +365,12 @@ long long link_capacity(const lbm_domain *D, const lbm_body &b) {
     return (long long)std::ceil(nodes) * (D->Q - 1) + 256;
 }
 
+// geometry chunks of a body whose region is ext
+int body_chunks(const lbm_domain *D, const int ext[3]) {
+    const int rows = geom_rows(D->p.nz);
+    return (int)(((long long)ext[1] * ext[2] + rows - 1) / rows);
+}
+
 void body_params(const lbm_domain *D, const lbm_body &b, BodyDev &o) {
     std::memset(&o, 0, sizeof(o));
     o.shape = b.shape;
@@ -372,8 +394,7 @@ void body_params(const lbm_domain *D, const lbm_body &b, BodyDev &o) {
         o.ext[a] = e;
     }
     long long vol = (long long)o.ext[0] * o.ext[1] * o.ext[2];
-    const int rows = geom_rows(D->p.nz);
-    o.nchunks = (int)(((long long)o.ext[1] * o.ext[2] + rows - 1) / rows);
+    o.nchunks = body_chunks(D, o.ext);
     o.link_cap = link_capacity(D, b);
     o.apm_cap = vol;
 }
@@ -1164,12 +1185,14 @@ int place_bodies(lbm_domain *D, const lbm_body *hb, int n) {
     D->p.me_stride = std::max<long long>(loff, 1);
     auto &T = D->body_allocs;
     const size_t nbx = (size_t)std::max(n, 1);
-    if ((rc = alloc_t(D, &D->dbodies, nbx, &T))) return rc;
+    const size_t nch = (size_t)std::max<long long>(chunks, 1);
+    if ((rc = alloc_t(D, &D->dbodies, nbx, &T, STATE_BODIES))) return rc;
     if ((rc = alloc_t(D, &D->dmoving, nbx, &T))) return rc;
-    if ((rc = alloc_t(D, &D->chunk_all, (size_t)std::max<long long>(chunks, 1), &T))) return rc;
-    if ((rc = alloc_t(D, &D->chunk_mov, (size_t)std::max<long long>(chunks, 1), &T))) return rc;
-    if ((rc = alloc_t(D, &D->chunk_cnt_apm, (size_t)std::max<long long>(chunks, 1), &T))) return rc;
-    if ((rc = alloc_t(D, &D->chunk_cnt_link, (size_t)std::max<long long>(chunks, 1), &T))) return rc;
+    if ((rc = alloc_t(D, &D->chunk_all, nch, &T, STATE_DERIVED))) return rc;
+    if ((rc = alloc_t(D, &D->chunk_mov, nch, &T, STATE_DERIVED))) return rc;
+    if ((rc = alloc_t(D, &D->chunk_cnt_apm, nch, &T, STATE_DERIVED))) return rc;
+    if ((rc = alloc_t(D, &D->chunk_cnt_link, nch, &T, STATE_DERIVED))) return rc;
+    D->chunk_cap = nch;
     // cut-link lists: FP64 mode and link mode (serving solves evaluate links
     // inside the boundary-node kernel); per-link contributions: FP64 mode
     const bool exact = D->prec == LBM_FP64;
@@ -1648,6 +1671,10 @@ int lbm_get_solid(lbm_domain *D, int32_t *out) {
 //
 // Layout: SnapHeader, the bodies as the host holds them (lbm_body, BodyDev),
 // the sizes of the device buffers, then their contents in allocation order.
+// The order never changes, so a snapshot of an earlier version can be read:
+// its bodies' records end before the FP32 record of served solves (which a
+// snapshot does not need), and its geometry chunks (BodyDev::nchunks, the
+// STATE_DERIVED buffers) are its own and made anew here.
 namespace {
 struct SnapHeader {
     char magic[8];
@@ -1657,13 +1684,50 @@ struct SnapHeader {
     int64_t nbuf;
 };
 constexpr char SNAP_MAGIC[8] = {'L', 'B', 'M', 'S', 'N', 'A', 'P', '1'};
+constexpr size_t SNAP_BODY_BYTES[] = {sizeof(BodyDev), offsetof(BodyDev, flf)}; // of this version, of earlier ones
+
+// offset of the buffer sizes in a snapshot whose body records have `rec` bytes
+int64_t snap_sizes_at(const SnapHeader &h, size_t rec) {
+    return (int64_t)sizeof(SnapHeader) + (int64_t)h.nb * (int64_t)(sizeof(lbm_body) + rec);
+}
+
+// whether a snapshot of `size` bytes is laid out for this domain with records of `rec` bytes
+bool snap_fits(const lbm_domain *D, const char *in, int64_t size, const SnapHeader &h, size_t rec,
+               std::vector<int64_t> &sizes) {
+    const int64_t list = snap_sizes_at(h, rec), count = (int64_t)D->state_bufs.size();
+    if (list + count * (int64_t)sizeof(int64_t) > size) return false;
+    sizes.resize((size_t)count);
+    std::memcpy(sizes.data(), in + list, (size_t)count * sizeof(int64_t));
+    int64_t end = list + count * (int64_t)sizeof(int64_t);
+    for (int64_t k = 0; k < count; ++k) {
+        const StateBuf &b = D->state_bufs[(size_t)k];
+        const int64_t n = sizes[(size_t)k];
+        if (n < 0 || n > size - end) return false;
+        if (b.kind == STATE_DATA && n != (int64_t)b.n) return false;
+        if (b.kind == STATE_BODIES && n != (int64_t)(b.n / sizeof(BodyDev) * rec)) return false;
+        end += n;
+    }
+    return end == size;
+}
+
+// the body records of a snapshot, with this version's chunks
+std::vector<BodyDev> snap_bodies(const lbm_domain *D, const char *at, size_t rec) {
+    std::vector<BodyDev> v((size_t)D->nb);
+    for (BodyDev &b : v) {
+        std::memset(&b, 0, sizeof(b));
+        std::memcpy(&b, at, rec);
+        b.nchunks = body_chunks(D, b.ext);
+        at += rec;
+    }
+    return v;
+}
 } // namespace
 
 int64_t lbm_state_bytes(const lbm_domain *D) {
     if (!D) return -1;
     int64_t b = (int64_t)sizeof(SnapHeader) + (int64_t)D->nb * (int64_t)(sizeof(lbm_body) + sizeof(BodyDev));
     b += (int64_t)D->state_bufs.size() * (int64_t)sizeof(int64_t);
-    for (const auto &e : D->state_bufs) b += (int64_t)e.second;
+    for (const auto &e : D->state_bufs) b += (int64_t)e.n;
     return b;
 }
 
@@ -1695,14 +1759,14 @@ int lbm_save_state(lbm_domain *D, void *out, int64_t cap) {
         p += sizeof(BodyDev) * D->nb;
     }
     for (const auto &e : D->state_bufs) {
-        const int64_t n = (int64_t)e.second;
+        const int64_t n = (int64_t)e.n;
         std::memcpy(p, &n, sizeof(n));
         p += sizeof(n);
     }
     for (const auto &e : D->state_bufs) {
-        CK(cudaMemcpy(p, e.first, e.second, cudaMemcpyDeviceToHost));
-        p += e.second;
-        D->d2h += (long long)e.second;
+        CK(cudaMemcpy(p, e.ptr, e.n, cudaMemcpyDeviceToHost));
+        p += e.n;
+        D->d2h += (long long)e.n;
     }
     return LBM_OK;
 }
@@ -1713,26 +1777,21 @@ int lbm_load_state(lbm_domain *D, const void *in, int64_t size) {
     const char *p = (const char *)in;
     SnapHeader h;
     std::memcpy(&h, p, sizeof(h));
-    p += sizeof(h);
     if (std::memcmp(h.magic, SNAP_MAGIC, 8) != 0) return fail(LBM_ERR_ARG, "not a domain snapshot");
     if (h.lattice != D->Q || h.precision != D->prec || h.nx != D->p.nx || h.ny != D->p.ny || h.nz != D->p.nz ||
-        h.nb != D->nb || h.nbuf != (int64_t)D->state_bufs.size() || size != lbm_state_bytes(D))
+        h.nb != D->nb || h.nbuf != (int64_t)D->state_bufs.size())
         return fail(LBM_ERR_ARG, "the snapshot belongs to a domain of another shape or body set");
+    std::vector<int64_t> sizes;
+    size_t rec = 0; // bytes of a body record
+    for (const size_t r : SNAP_BODY_BYTES)
+        if (rec == 0 && snap_fits(D, p, size, h, r, sizes)) rec = r;
+    if (rec == 0) return fail(LBM_ERR_ARG, "the snapshot's buffers do not match this domain's");
     std::vector<lbm_body> hb((size_t)D->nb);
-    std::vector<BodyDev> hbd((size_t)D->nb);
-    if (D->nb) {
-        std::memcpy(hb.data(), p, sizeof(lbm_body) * D->nb);
-        p += sizeof(lbm_body) * D->nb;
-        std::memcpy(hbd.data(), p, sizeof(BodyDev) * D->nb);
-        p += sizeof(BodyDev) * D->nb;
-    }
-    for (size_t k = 0; k < D->state_bufs.size(); ++k) {
-        int64_t n;
-        std::memcpy(&n, p, sizeof(n));
-        p += sizeof(n);
-        if (n != (int64_t)D->state_bufs[k].second)
-            return fail(LBM_ERR_ARG, "the snapshot's buffers do not match this domain's");
-    }
+    std::memcpy(hb.data(), p + sizeof(h), sizeof(lbm_body) * (size_t)D->nb);
+    std::vector<BodyDev> hbd = snap_bodies(D, p + sizeof(h) + sizeof(lbm_body) * (size_t)D->nb, rec);
+    long long chunks = 0;
+    for (const BodyDev &b : hbd) chunks += std::max(b.nchunks, 0);
+    if (chunks > (long long)D->chunk_cap) return fail(LBM_ERR_ARG, "the snapshot's bodies do not match this domain's");
     CK(cudaStreamSynchronize(D->s));
     if (D->nb) { // the host's body records and the body maps they imply, then the device state over them
         D->hb = hb;
@@ -1740,10 +1799,18 @@ int lbm_load_state(lbm_domain *D, const void *in, int64_t size) {
         int rc = upload_bodies(D);
         if (rc) return rc;
     }
-    for (const auto &e : D->state_bufs) {
-        CK(cudaMemcpy(e.first, p, e.second, cudaMemcpyHostToDevice));
-        p += e.second;
-        D->h2d += (long long)e.second;
+    p += snap_sizes_at(h, rec) + (int64_t)(sizes.size() * sizeof(int64_t));
+    for (size_t k = 0; k < sizes.size(); ++k) {
+        const StateBuf &e = D->state_bufs[k];
+        if (e.kind == STATE_DATA) {
+            CK(cudaMemcpy(e.ptr, p, e.n, cudaMemcpyHostToDevice));
+            D->h2d += (long long)e.n;
+        } else if (e.kind == STATE_BODIES && D->nb) { // (free bodies: not the host's)
+            const std::vector<BodyDev> dev = snap_bodies(D, p, rec);
+            CK(cudaMemcpy(e.ptr, dev.data(), sizeof(BodyDev) * dev.size(), cudaMemcpyHostToDevice));
+            D->h2d += (long long)(sizeof(BodyDev) * dev.size());
+        }
+        p += sizes[k];
     }
     D->t = h.t;
     D->prep_dirty = h.prep_dirty != 0;
@@ -1752,6 +1819,18 @@ int lbm_load_state(lbm_domain *D, const void *in, int64_t size) {
     D->ev_used = 0;
     D->g_timed = false;
     for (int k = 0; k < lbm_domain::N_STEP_EV; ++k) D->step_ev_t[k] = -1;
+    if (rec != sizeof(BodyDev) && D->nb) { // an earlier version's state
+        D->prep_dirty = true; // its link tiles had another size
+        if (D->prec == LBM_FP64) {
+            // moments were kept within two links of a body only, and the covered /
+            // uncovered lists (explicit scheme) were applied to the flags by the
+            // step that made them
+            CK(launch_macband(D->p, geom_args(D, false), D->s));
+            if (D->p.free_scheme == LBM_FREE_EXPLICIT)
+                CK(cudaMemsetAsync(D->apm_cnt, 0, sizeof(long long) * (size_t)D->nb, D->s));
+            CK(cudaStreamSynchronize(D->s));
+        }
+    }
     return LBM_OK;
 }
 
