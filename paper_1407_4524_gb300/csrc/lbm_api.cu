@@ -135,7 +135,7 @@ struct DevGuard {
 enum StateKind {
     STATE_DATA,    // its contents, of the same size in every version of the library
     STATE_BODIES,  // the bodies' records, which have grown
-    STATE_DERIVED, // made anew from the bodies' records: contents and size are the writer's own
+    STATE_DERIVED, // made anew from the bodies' records, or not read back: contents and size are the writer's own
 };
 struct StateBuf {
     void *ptr;
@@ -199,11 +199,9 @@ struct lbm_domain {
     uint8_t *chg_val = nullptr;
     long long chg_cap = 0;
     uint32_t *bn_static = nullptr;
-    uint32_t *bn_mov[2] = {nullptr, nullptr};
-    unsigned long long *bn_cnt = nullptr; // [0] static, [1], [2] moving lists of even / odd steps
-    long long bn_static_cap = 0, bn_mov_cap = 0;
+    unsigned long long *bn_cnt = nullptr; // length of bn_static
+    long long bn_static_cap = 0;
     bool lists_dirty = true;
-    int bnd_grid = 0, bnd_grid_full = 0;
     int side_blocks = 0; // block cap of the side-stream kernels
     bool side_serial = false; // run the surface kernels before k_bulk on one stream, uncapped
     bool tma = false;         // the stream-collide pass is the persistent kernel on bulk-copied tiles
@@ -293,6 +291,8 @@ void free_body_buffers(lbm_domain *D) {
             }
         D->release(ptr);
     }
+    D->state_bufs.erase(std::remove_if(D->state_bufs.begin(), D->state_bufs.end(), [](const StateBuf &b) { return !b.ptr; }),
+                        D->state_bufs.end());
     D->body_allocs.clear();
     for (int k = 0; k < 2; ++k) { // pinned body staging: sized for the body count it was made for
         if (!D->hbd_pin[k]) continue;
@@ -328,9 +328,8 @@ void free_body_buffers(lbm_domain *D) {
     D->chg_val = nullptr;
     D->chg_cap = 0;
     D->bn_static = nullptr;
-    D->bn_mov[0] = D->bn_mov[1] = nullptr;
     D->bn_cnt = nullptr;
-    D->bn_static_cap = D->bn_mov_cap = 0;
+    D->bn_static_cap = 0;
     D->lists_dirty = true;
     D->prep_dirty = true;
     D->nb = D->n_moving = D->n_free = 0;
@@ -523,10 +522,7 @@ GeomArgs geom_args(lbm_domain *D, bool moving_step) {
     g.chg_cap = D->chg_cap;
     g.bn_static = D->bn_static;
     g.bn_static_cnt = D->bn_cnt;
-    g.bn_mov = D->bn_mov[nxt];
-    g.bn_mov_cnt = D->bn_cnt + 1 + nxt;
     g.bn_static_cap = D->bn_static_cap;
-    g.bn_mov_cap = D->bn_mov_cap;
     // FP64 mode, semi-implicit schemes (one stream): the node flags follow the
     // geometry; elsewhere the kept-moment band only gains flags (linkmode, or
     // geom_a in FP64 mode)
@@ -617,18 +613,10 @@ int upload_bodies(lbm_domain *D) {
     return LBM_OK;
 }
 
-// reduced-precision modes: boundary-node lists of step t from scratch
+// served solves: the boundary-node list of their (static) bodies
 int build_bnd_lists(lbm_domain *D) {
-    if (D->p.linkmode) { // link mode keeps cut-link lists instead
-        D->lists_dirty = false;
-        return LBM_OK;
-    }
-    const int cur = (int)(D->t & 1);
-    CK(cudaMemsetAsync(D->bn_cnt, 0, 3 * sizeof(unsigned long long), D->s));
-    GeomArgs gl = geom_args(D, false);
-    gl.bn_mov = D->bn_mov[cur];
-    gl.bn_mov_cnt = D->bn_cnt + 1 + cur;
-    CK(launch_bnd_lists(D->Q, D->p, gl, D->s));
+    CK(cudaMemsetAsync(D->bn_cnt, 0, sizeof(unsigned long long), D->s));
+    CK(launch_bnd_lists(D->Q, D->p, geom_args(D, false), D->s));
     D->lists_dirty = false;
     return LBM_OK;
 }
@@ -735,8 +723,7 @@ int prepare_step(lbm_domain *D) {
                            D->apm_cnt, D->apm_cell, D->apm_sign, D->s));
     } else if (D->n_moving || D->prep_dirty || D->lists_dirty) {
         CK(launch_fprep(D->p, D->dbodies, D->poses, D->t, tdev, D->flags, D->chg_cnt, D->chg_cell, D->chg_val,
-                        D->chg_cap, D->apm_cnt, D->bn_cnt + 1 + nxt, D->link_cnt[cur], D->link_cnt[nxt], D->tile_pre,
-                        D->s));
+                        D->chg_cap, D->apm_cnt, D->link_cnt[cur], D->link_cnt[nxt], D->tile_pre, D->s));
     }
     D->prep_dirty = false;
     D->lists_dirty = false;
@@ -1208,7 +1195,7 @@ int place_bodies(lbm_domain *D, const lbm_body *hb, int n) {
     if ((rc = alloc_t(D, &D->apm_cell, (size_t)std::max<long long>(aoff, 1), &T))) return rc;
     if ((rc = alloc_t(D, &D->apm_sign, (size_t)std::max<long long>(aoff, 1), &T))) return rc;
     if ((rc = alloc_t(D, &D->apm_cnt, nbx, &T))) return rc;
-    if ((rc = alloc_t(D, &D->imp_prev, nbx * 6, &T))) return rc; // zero: no displacement before t = 0
+    if ((rc = alloc_t(D, &D->imp_prev, D->batch ? 0 : nbx * 6, &T))) return rc; // zero: no displacement before t = 0
     if (D->p.free_scheme == LBM_FREE_PREDICTOR) {
         if ((rc = alloc_t(D, &D->apm_pred_cell, (size_t)std::max<long long>(aoff, 1), &T))) return rc;
         if ((rc = alloc_t(D, &D->apm_pred_sign, (size_t)std::max<long long>(aoff, 1), &T))) return rc;
@@ -1223,27 +1210,16 @@ int place_bodies(lbm_domain *D, const lbm_body *hb, int n) {
     if ((rc = alloc_t(D, &D->chg_cnt, 1, &T))) return rc;
     if ((rc = alloc_t(D, &D->chg_cell, (size_t)D->chg_cap, &T))) return rc;
     if ((rc = alloc_t(D, &D->chg_val, (size_t)D->chg_cap, &T))) return rc;
-    // boundary nodes of a body lie in the shell R < |x - X| <= R + sqrt(2):
+    // served solves: boundary nodes of a body lie in the shell R < |x - X| <= R + sqrt(2):
     // link_cap / (Q - 1) bounds their number (see link_capacity)
-    long long bns = 0, bnm = 0;
-    for (int b = 0; b < n; ++b) {
-        const long long nodes = D->hbd[b].link_cap / (D->Q - 1) + 64;
-        bns += nodes;
-        if (D->hbd[b].moving) bnm += nodes;
-    }
+    long long bns = 0;
+    if (D->batch)
+        for (int b = 0; b < n; ++b) bns += D->hbd[b].link_cap / (D->Q - 1) + 64;
     D->bn_static_cap = std::max<long long>(bns, 1);
-    D->bn_mov_cap = std::max<long long>(bns, 1); // bodies may start moving later
-    (void)bnm;
-    if ((rc = alloc_t(D, &D->bn_static, (size_t)D->bn_static_cap, &T))) return rc;
-    if ((rc = alloc_t(D, &D->bn_mov[0], (size_t)D->bn_mov_cap, &T))) return rc;
-    if ((rc = alloc_t(D, &D->bn_mov[1], (size_t)D->bn_mov_cap, &T))) return rc;
-    if ((rc = alloc_t(D, &D->bn_cnt, 3, &T))) return rc;
-    D->bnd_grid = (int)std::max<long long>(1, std::min<long long>(D->side_blocks, (bns + 7) / 8));
-    D->bnd_grid_full = (int)std::max<long long>(1, std::min<long long>(16ll * D->p.nsm, (bns + 7) / 8));
+    if ((rc = alloc_t(D, &D->bn_static, (size_t)D->bn_static_cap, &T, STATE_DERIVED))) return rc;
+    for (int k = 0; k < 2; ++k) D->state_bufs.push_back({nullptr, 0, STATE_DERIVED}); // (two lists that earlier versions kept)
+    if ((rc = alloc_t(D, &D->bn_cnt, 1, &T, STATE_DERIVED))) return rc;
     D->lists_dirty = true;
-    long long maxcnt = 0;
-    for (int b = 0; b < n; ++b) maxcnt = std::max(maxcnt, D->hbd[b].link_cap);
-    (void)maxcnt;
     D->links_grid = (int)std::max<long long>(1, std::min<long long>(16 * 152, tiles_cap));
     if ((rc = upload_bodies(D))) return rc;
 
@@ -1764,7 +1740,7 @@ int lbm_save_state(lbm_domain *D, void *out, int64_t cap) {
         p += sizeof(n);
     }
     for (const auto &e : D->state_bufs) {
-        CK(cudaMemcpy(p, e.ptr, e.n, cudaMemcpyDeviceToHost));
+        if (e.n) CK(cudaMemcpy(p, e.ptr, e.n, cudaMemcpyDeviceToHost));
         p += e.n;
         D->d2h += (long long)e.n;
     }
@@ -1915,7 +1891,7 @@ int lbm_kernel_time(lbm_domain *D, int64_t *launches, double *total_ms) {
 int lbm_launches_per_step(const lbm_domain *D, int *out) {
     if (!D || !out) return fail(LBM_ERR_ARG, "invalid arguments");
     if (D->prec != LBM_FP64 && D->nb)
-        *out = 3 + (D->n_moving ? 3 : (D->prep_dirty ? 1 : 0)); // bulk, bnd, finish (+ prep, geometry)
+        *out = 3 + (D->n_moving ? 3 : (D->prep_dirty ? 1 : 0)); // links, bulk, finish (+ prep, geometry)
     else
         *out = 1 + (D->nb ? 2 : 0) + (D->n_moving ? 4 : 0) + (D->nb && D->prep_dirty && !D->n_moving ? 1 : 0);
     if (D->n_free) *out += 1; // free-body update
@@ -2046,12 +2022,11 @@ int domain_bytes(const lbm_domain_desc &d, const lbm_body *hb, int n, int64_t *b
     b += 2 * (Lsz * 4 + Lsz * 1 + Lsz * 8 + nbx * 8);            // link lists and counts
     b += Lsz * ME_PER_LINK * 8;                                  // per-link contributions
     b += A * 4 + A * 1 + nbx * 8;                                // covered/uncovered lists
-    b += nbx * 6 * 8;                                            // impulsive terms of the last displacement
     if (d.free_scheme == LBM_FREE_PREDICTOR) b += A * 4 + A * 1 + nbx * 8; // predicted lists
     b += cap * nbx * SERIES_ROW * 8 + nbx * POSE_STRIDE * 8;     // series, poses
     b += 2 * (nbx + 1) * 8 + nbx * SERIES_ROW * 8;               // prefixes, accumulators
     b += 8 + A * 4 + A * 1;                                      // flag-change list
-    b += B * 4 * 3 + 3 * 8;                                      // boundary-node lists
+    b += B * 4 + 8;                                              // boundary-node list
     *bytes = b;
     return LBM_OK;
 }
@@ -2331,7 +2306,7 @@ int lbm_batch_admit(lbm_batch *B, const lbm_domain_desc *desc, const lbm_body *h
     if (n > 0) {
         // poses of t = 0 and the boundary-node list (all static)
         cudaError_t e = launch_fprep(D->p, D->dbodies, D->poses, 0, nullptr, D->flags, D->chg_cnt, D->chg_cell, D->chg_val,
-                                     D->chg_cap, D->apm_cnt, D->bn_cnt + 2, nullptr, nullptr, nullptr, D->s);
+                                     D->chg_cap, D->apm_cnt, nullptr, nullptr, nullptr, D->s);
         if (e == cudaSuccess) e = launch_body_f32(D->p, D->dbodies, D->poses, D->s);
         if (e == cudaSuccess && (rc = build_bnd_lists(D))) {
             lbm_destroy_domain(D);

@@ -367,17 +367,6 @@ __global__ void k_export(Params p, const typename P::S *pop, double *out) {
     }
 }
 
-template <class L, class P>
-__global__ void k_import(Params p, const double *in, typename P::S *pop) {
-    const long long n = (long long)L::Q * p.N;
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(k / p.N);
-        double v = in[k];
-        if constexpr (!P::exact) v -= L::template w<double>(i);
-        stS(pop + k, (typename P::C)v);
-    }
-}
-
 
 // ----------------------------------------------------------------------------
 // Reduced-precision modes.  Momentum-exchange sums are order independent
@@ -391,8 +380,8 @@ __global__ void __launch_bounds__(1024) k_fprep(Params p, const BodyDev *bodies,
                                                 const unsigned long long *tdev, uint8_t *flags,
                                                 unsigned long long *chg_cnt, const uint32_t *chg_cell,
                                                 const uint8_t *chg_val, long long chg_cap, long long *apm_cnt,
-                                                unsigned long long *bn_mov_next_cnt, const long long *link_cnt_t,
-                                                long long *link_cnt_t1, long long *tile_pre) {
+                                                const long long *link_cnt_t, long long *link_cnt_t1,
+                                                long long *tile_pre) {
     if (blockIdx.x == 0) {
         if (p.linkmode && link_cnt_t) {
             // link mode: the cut links of t are complete (static bodies: from
@@ -412,10 +401,7 @@ __global__ void __launch_bounds__(1024) k_fprep(Params p, const BodyDev *bodies,
             flags[c] = (uint8_t)((flags[c] & ~(FL_SOLID | FL_BND)) | chg_val[e]);
         }
         __syncthreads(); // every thread has read the count
-        if (threadIdx.x == 0) {
-            *chg_cnt = 0ull;
-            *bn_mov_next_cnt = 0ull;
-        }
+        if (threadIdx.x == 0) *chg_cnt = 0ull;
         return;
     }
     const long long t = tdev ? (long long)*tdev : t_arg; // the device step counter, when given
@@ -534,9 +520,8 @@ __global__ void __launch_bounds__(GEOM_THREADS, GEOM_MIN_BLOCKS) k_fgeom2l(Param
     }
 }
 
-// boundary-node lists of step t from scratch: nodes next only to static
-// bodies go to the static list, nodes next to a moving body to the moving
-// list of step t (each node once: by the lowest-numbered neighbour body)
+// served solves, at admission: the nodes next to a body (each node once: by the
+// lowest-numbered neighbour body)
 template <class L>
 __global__ void __launch_bounds__(GEOM_THREADS) k_bnd_lists(Params p, GeomArgs g) {
     __shared__ ShellChunk c;
@@ -550,21 +535,14 @@ __global__ void __launch_bounds__(GEOM_THREADS) k_bnd_lists(Params p, GeomArgs g
         const RegionCell rc = shell_cell(p, c, e);
         const float dist = frame_dist(p, B, c.F, rc);
         if (dist < Rin - 0.5f || dist > Rout + 1.5f || g.owner_t[rc.cell] != 0) continue;
-        int minall = 1 << 20, minmov = 1 << 20;
+        int lowest = 1 << 20;
 #pragma unroll
         for (int i = 1; i < L::Q; ++i) {
             const long long a = nbr<L>(p, rc.x, rc.y, rc.z, i, 1);
             const unsigned o = a >= 0 ? g.owner_t[a] : 0u;
-            if (!o) continue;
-            minall = min(minall, (int)o);
-            if (g.bodies[o - 1].moving) minmov = min(minmov, (int)o);
+            if (o) lowest = min(lowest, (int)o);
         }
-        if (minmov < (1 << 20)) {
-            if (minmov == b + 1) {
-                const unsigned long long at = atomicAdd(g.bn_mov_cnt, 1ull);
-                if ((long long)at < g.bn_mov_cap) g.bn_mov[at] = (uint32_t)rc.cell;
-            }
-        } else if (minall == b + 1) {
+        if (lowest == b + 1) {
             const unsigned long long at = atomicAdd(g.bn_static_cnt, 1ull);
             if ((long long)at < g.bn_static_cap) g.bn_static[at] = (uint32_t)rc.cell;
         }
@@ -605,10 +583,9 @@ cudaError_t launch_prep(const Params &p, const BodyDev *bodies, const long long 
 cudaError_t launch_fprep(const Params &p, const BodyDev *bodies, double *poses, long long t,
                          const unsigned long long *tdev, uint8_t *flags, unsigned long long *chg_cnt,
                          const uint32_t *chg_cell, const uint8_t *chg_val, long long chg_cap, long long *apm_cnt,
-                         unsigned long long *bn_mov_next_cnt, const long long *link_cnt_t, long long *link_cnt_t1,
-                         long long *tile_pre, cudaStream_t s) {
+                         const long long *link_cnt_t, long long *link_cnt_t1, long long *tile_pre, cudaStream_t s) {
     k_fprep<<<3, 1024, 0, s>>>(p, bodies, poses, t, tdev, flags, chg_cnt, chg_cell, chg_val, chg_cap, apm_cnt,
-                               bn_mov_next_cnt, link_cnt_t, link_cnt_t1, tile_pre);
+                               link_cnt_t, link_cnt_t1, tile_pre);
     return cudaGetLastError();
 }
 
@@ -703,15 +680,6 @@ static cudaError_t export_t(int prec, const Params &p, const void *pop, double *
     return cudaGetLastError();
 }
 
-template <class L>
-static cudaError_t import_t(int prec, const Params &p, const double *in, void *pop, cudaStream_t s) {
-    const int grid = 4 * 152;
-    if (prec == 0) k_import<L, PF64><<<grid, 256, 0, s>>>(p, in, (double *)pop);
-    else if (prec == 1) k_import<L, PF32><<<grid, 256, 0, s>>>(p, in, (float *)pop);
-    else k_import<L, PF16><<<grid, 256, 0, s>>>(p, in, (__half *)pop);
-    return cudaGetLastError();
-}
-
 // Free bodies (one thread per body), after the force/torque row of step t is
 // complete.  Explicit scheme: the pose advances with U(t) -- the motion the
 // step's A+/A- sets were built from.  Semi-implicit schemes (the row holds the
@@ -803,10 +771,6 @@ cudaError_t launch_pose1(const Params &p, const BodyDev *bodies, double *poses, 
 
 cudaError_t launch_export(int Q, int prec, const Params &p, const void *pop, double *out, cudaStream_t s) {
     return Q == 9 ? export_t<Lat<9>>(prec, p, pop, out, s) : export_t<Lat<19>>(prec, p, pop, out, s);
-}
-
-cudaError_t launch_import(int Q, int prec, const Params &p, const double *in, void *pop, cudaStream_t s) {
-    return Q == 9 ? import_t<Lat<9>>(prec, p, in, pop, s) : import_t<Lat<19>>(prec, p, in, pop, s);
 }
 
 } // namespace lbm

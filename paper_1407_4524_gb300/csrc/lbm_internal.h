@@ -36,13 +36,10 @@ struct GeomArgs {
     uint32_t *chg_cell;
     uint8_t *chg_val;
     long long chg_cap;
-    // reduced-precision modes: boundary-node lists (static bodies; moving
-    // bodies of the step being built)
+    // served solves: boundary-node list
     uint32_t *bn_static;
     unsigned long long *bn_static_cnt;
-    uint32_t *bn_mov;
-    unsigned long long *bn_mov_cnt;
-    long long bn_static_cap, bn_mov_cap;
+    long long bn_static_cap;
     int grid_cap; // > 0: at most this many blocks (side-stream kernels)
 };
 
@@ -89,8 +86,7 @@ cudaError_t launch_prep(const Params &p, const BodyDev *bodies, const long long 
 cudaError_t launch_fprep(const Params &p, const BodyDev *bodies, double *poses, long long t,
                          const unsigned long long *tdev, uint8_t *flags, unsigned long long *chg_cnt,
                          const uint32_t *chg_cell, const uint8_t *chg_val, long long chg_cap, long long *apm_cnt,
-                         unsigned long long *bn_mov_next_cnt, const long long *link_cnt_t, long long *link_cnt_t1,
-                         long long *tile_pre, cudaStream_t s);
+                         const long long *link_cnt_t, long long *link_cnt_t1, long long *tile_pre, cudaStream_t s);
 // served solves: the FP32 record of each (static) body
 cudaError_t launch_body_f32(const Params &p, BodyDev *bodies, const double *poses, cudaStream_t s);
 // link mode: FL_MAC on the nodes within R + MAC_BAND of every body at t
@@ -132,6 +128,5 @@ cudaError_t launch_pose1(const Params &p, const BodyDev *bodies, double *poses, 
 
 // population export: fhat as FP64 f (adds w back for the shifted modes)
 cudaError_t launch_export(int Q, int prec, const Params &p, const void *pop, double *out, cudaStream_t s);
-cudaError_t launch_import(int Q, int prec, const Params &p, const double *in, void *pop, cudaStream_t s);
 
 } // namespace lbm

@@ -962,7 +962,7 @@ __device__ __forceinline__ void bulk_node(const Params &p, const typename P::S *
         if (fl & FL_SOLID) return;
     }
     // reduced precision: the pulls do not wait for the flag (a solid node, or
-    // a boundary node left to k_bnd, is stepped and not stored), so the flag
+    // a served boundary node left to k_bbnd, is stepped and not stored), so the flag
     // load and the population loads are in flight together
     bool store = true;
     if constexpr (!P::exact) store = !(fl & FL_SOLID) && (p.linkmode || !(fl & FL_BND));
