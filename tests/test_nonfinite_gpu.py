@@ -42,20 +42,22 @@ def test_macros_of_overflowed_populations(lattice, n, eq):
     assert np.isposinf(got[1].ravel()[3]) == (eq == "incomp") and np.isnan(got[2].ravel()[3])
 
 
+@pytest.mark.parametrize("edges", [{"y": ("wall", "wall")}, {"x": ("wall", "wall")}, {"x": ("wall", "outlet")}])
 @pytest.mark.parametrize("lattice,n", [("D2Q9", (9, 7)), ("D3Q19", (6, 5, 7))])
-def test_resting_wall_of_an_overflowed_node(lattice, n):
+def test_resting_wall_of_an_overflowed_node(lattice, n, edges):
     """Standard model: a wall link at rest adds 6 w_i rho (c_i . u_B) with u_B =
     0 and the node's own density, so a node whose density overflowed has no
     finite population after the step."""
     from paper_1407_4524_gb300 import lbm
-    dom = lbm.Domain(dict(lattice=lattice, n=n, tau=1e7, eq="standard", precision="fp16",
-                          edges={"y": ("wall", "wall")}), device=0)
+    dom = lbm.Domain(dict(lattice=lattice, n=n, tau=1e7, eq="standard", precision="fp16", edges=edges), device=0)
     f = dom.populations()
-    f.reshape(f.shape[0], -1)[1, 3] = 1e5  # a node of the y-low wall row; leaves along +x
+    # a node of the y-low (x-low) wall row; its large population leaves along +x (+y)
+    i, at, to, away = (1, 3, 4, 2) if "y" in edges else (2 if lattice == "D2Q9" else 3, n[0], 2 * n[0], 0)
+    f.reshape(f.shape[0], -1)[i, at] = 1e5
     dom.set_populations(f)
     before = dom.populations().reshape(f.shape[0], -1)
-    assert np.isposinf(before[1, 3]) and np.isfinite(np.delete(before, 1, 0)).all()
+    assert np.isposinf(before[i, at]) and np.isfinite(np.delete(before, i, 0)).all()
     dom.step(1)
     after = dom.populations().reshape(f.shape[0], -1)
-    assert np.isnan(after[:, 3]).all()
-    assert not np.isfinite(after[:, 4]).any() and np.isfinite(after[:, 2]).all()
+    assert np.isnan(after[:, at]).all()
+    assert not np.isfinite(after[:, to]).any() and np.isfinite(after[:, away]).all()
