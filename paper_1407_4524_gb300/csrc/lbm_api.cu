@@ -1573,7 +1573,8 @@ int lbm_get_macros(lbm_domain *D, double *out) {
     const long long N = D->p.N, chunk = N <= IO_CHUNK / 2 ? N : std::min(IO_CHUNK / 2, (N + 1) / 2);
     const long long chunks = (N + chunk - 1) / chunk;
     PageToucher pages;
-    double *stage = (double *)D->alloc((size_t)(chunks > 1 ? 2 : 1) * chunk * 4 * sizeof(double));
+    // (the second half of two chunks holds the shorter one: never more than min(N, IO_CHUNK) cells)
+    double *stage = (double *)D->alloc((size_t)std::min(2 * chunk, N) * 4 * sizeof(double));
     if (!stage) return fail(LBM_ERR_OOM, "temporary staging buffer");
     cudaEvent_t done[2] = {nullptr, nullptr};
     cudaError_t e = cudaSuccess;
