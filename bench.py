@@ -440,7 +440,7 @@ def run_serving(args, dev):
 # the sources that define the stream-collide kernel and its launch (the
 # kernel the traffic figure belongs to)
 BULK_SOURCES = ("lbm_dev.cuh", "lbm_step.cuh", "lbm_pair.cuh", "lbm_launch.cuh", "lbm_stage.cuh", "lbm_tma.cuh",
-                "lbm_fp32.cu", "lbm_fp64.cu")
+                "lbm_fp32.cu", "lbm_fp64.cu", "lbm_cols.h", "lbm_wait.h")
 
 
 def _kernel_rev() -> str:

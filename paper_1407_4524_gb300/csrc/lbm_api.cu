@@ -6,11 +6,11 @@
 // per-link momentum-exchange contributions, the covered/uncovered lists and
 // the force/torque ring.  lbm_step enqueues, per step (do_step):
 //   main stream: k_prep / k_fprep (poses, solid flags, link prefixes), k_links
-//   (wall values + ME per link), k_bulk / k_bulk_pair (stream-collide; then
-//   k_zouhe for the Zou-He face nodes);
-//   high-priority side stream, beside the stream-collide pass: k_geom_a/b/c or
-//   k_fgeom1/2l (geometry of t+1, moving bodies), k_finish (per-body series
-//   row; A+/A- impulsive terms and refill), k_free (free bodies).
+//   (wall values + ME per link), k_bulk / k_bulk_pair / k_bulk_tma (stream-collide);
+//   two side streams beside the pass: k_geom_a/b or k_fgeom1 (owners of t+1,
+//   moving bodies), k_finish (per-body series row; A+/A- impulsive terms and
+//   refill) and k_free (free bodies) on one, k_zouhe (Zou-He face nodes) and
+//   k_geom_c or k_fgeom2l (cut links of t+1) on the other.
 // Each lbm_step call ends with a step event that the series reads wait on.
 // The serving batch (lbm_batch_*) keeps solves of this kind in slots and
 // replays a CUDA graph of batched ticks (lbm_batch.cu).  Every persistent
@@ -211,8 +211,8 @@ struct lbm_domain {
     // planes without cut links, the longest run of them (static bodies in 3-D; 0: none worth it)
     int split_z0 = 0, split_n = 0;
     int64_t t = 0;
-    // side stream: in the reduced-precision modes the geometry of t+1 and the
-    // end-of-step kernel run on it, concurrently with the bulk kernel
+    // side streams: the geometry of t+1, the Zou-He face nodes and the end-of-step
+    // kernels run on them beside the stream-collide pass (do_step)
     cudaStream_t s2 = nullptr, s3 = nullptr;
     cudaEvent_t ev_prep = nullptr, ev_links = nullptr, ev_side = nullptr, ev_own = nullptr, ev_third = nullptr;
     // timing of the bulk kernel

@@ -62,6 +62,8 @@ __device__ __forceinline__ long long block_sum_range(const int *cnt, int first, 
     return r;
 }
 
+// store macros at x if x is fluid and within two hops of a solid node (the
+// fluid end of a cut link, or its u_G node), or on a non-periodic face
 template <class L>
 __device__ __forceinline__ uint8_t node_flags(const Params &p, const uint16_t *owner_t, const uint16_t *owner_m,
                                               int x, int y, int z, long long cell) {

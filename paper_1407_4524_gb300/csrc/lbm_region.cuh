@@ -170,8 +170,7 @@ __device__ __forceinline__ bool edge_node(const Params &p, int x, int y, int z) 
            (!p.per[2] && (z == 0 || z == p.nz - 1));
 }
 
-// store macros at x if x is fluid and within two hops of a solid node (the
-// fluid end of a cut link, or its u_G node), or on a non-periodic face
+// distance of a cell from the axis or centre of a body (FP32 frame)
 __device__ __forceinline__ float frame_dist(const Params &p, const BodyDev &B, const Frame &F, const RegionCell &rc) {
     float d[3];
     frame_disp_f(p, F, rc.x, rc.y, rc.z, d);

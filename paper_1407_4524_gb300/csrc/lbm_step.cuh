@@ -168,7 +168,7 @@ __device__ __forceinline__ void collide_all_x(const Params &p, double f[], doubl
 // whatever the two directions i, opp(i) of a pair share (c_o . u = -(c_i . u)
 // exactly: rounding to nearest is symmetric).  Every remaining operation and
 // its order are those of the *_all_x forms, so the results are the same bits.
-// D3Q19: 216 FP64 operations a node instead of 437 and three divisions; the
+// D3Q19: 219 FP64 operations a node instead of some 440 and three divisions; the
 // 256x128x128 sphere channel's step 3.66 -> 2.49 ms, the 200x80 cylinder
 // channel's 38.8 -> 31.0 us.
 template <class L>

@@ -6,14 +6,15 @@
 // moments need them, at eight blocks of 128 threads an SM (45 % of the warps):
 // 0.78 of the measured copy rate on the 512x256x256 swarm, 0.59 on the
 // 256x128x128 channel, whose x faces the direct kernels step one node a thread.
-// This one: 0.89 (424 us, bound by DRAM) and 0.80 (59 us, 5 of them filling and
-// draining the ring); instructions a node 281 -> 242.
+// This one: 0.93 (403 us in the step, bound by DRAM) and 0.80 (59 us, 5 of them
+// filling and draining the ring); instructions a node 275 -> 241.
 // Here a block takes a tile of TY whole rows of one plane z.  Whole rows are
 // contiguous, so the sources of direction i -- rows y - c_iy of plane z - c_iz
 // of population i -- are one copy of TY * nx values (two where the tile meets
 // the periodic y seam), and the x shift and its periodic wrap are an index into
 // the row.  Up to TMA_STAGES tiles of 19 copies are in flight per SM (nothing
-// of that in registers), issued by a producer warp; the others wait for a tile, takes its two nodes a lane, releases the stage and goes on with
+// of that in registers), issued by a producer warp.  Each other warp waits for
+// a tile, takes two nodes a lane, releases the stage and goes on with
 // moments_pair / collide_pair: the operations of the direct kernels, so the
 // same values.
 //
@@ -40,7 +41,7 @@ template <class S> __host__ __device__ constexpr int tma_threads() { return tma_
 // registers, so that an SM sub-partition's five warps leave space for the two
 // warps of a geometry block (48 registers) and the side stream runs beside the
 // pass; the 96 registers the kernel takes otherwise keep it out until the end
-// (512x256x256 swarm: step 0.557 ms against 0.468), and are 4 % faster where
+// (512x256x256 swarm: step 0.488 ms against 0.437), and are 4 % faster where
 // there is no geometry (256x128x128 channel)
 template <class S, bool ROOM> __host__ __device__ constexpr int tma_reg_threads() { return ROOM ? 768 : tma_threads<S>(); }
 
